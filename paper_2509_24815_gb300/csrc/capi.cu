@@ -388,24 +388,23 @@ int exact_impl(seismic_index *ix, const seismic_csr *queries, uint32_t k, uint32
     d_ids = w->out.as<uint32_t>();
     d_sc = reinterpret_cast<float *>(d_ids + (size_t)nq * k);
   }
-  uint32_t grid = (uint32_t)std::min<uint64_t>(nq, 2ull * sm_count(ix->device));
-  size_t accb = (size_t)grid * ix->n_docs * 4;
-  if ((rc = ix->ws_exact.ensure(accb))) return rc;
-  SZ_CUDA(cudaMemsetAsync(ix->ws_exact.p, 0, accb, st));
   ExactArgs a{};
   a.full_ptr = ix->full_ptr.as<uint32_t>();
   a.full_doc = ix->full_doc.as<uint32_t>();
   a.full_val = ix->full_val.as<float>();
   a.n_docs = (uint32_t)ix->n_docs;
+  a.dim = ix->dim;
   a.q_indptr = q.ip;
   a.q_terms = q.t;
   a.q_vals = q.v;
   a.nq = nq;
   a.k = k;
-  a.acc = ix->ws_exact.as<float>();
   a.ids = d_ids;
   a.scores = d_sc;
-  if ((rc = launch_exact(a, grid, st))) return rc;
+  const uint32_t sms = (uint32_t)sm_count(ix->device);
+  if ((rc = ix->ws_exact.ensure(exact_layout(a, sms, nullptr)))) return rc;
+  exact_layout(a, sms, ix->ws_exact.p);
+  if ((rc = launch_exact(a, st))) return rc;
   if (!out_on_device) {
     SZ_CUDA(cudaMemcpyAsync(ids_out, d_ids, (size_t)nq * k * 4, cudaMemcpyDeviceToHost, st));
     SZ_CUDA(cudaMemcpyAsync(scores_out, d_sc, (size_t)nq * k * 4, cudaMemcpyDeviceToHost, st));

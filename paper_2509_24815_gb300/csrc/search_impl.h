@@ -87,17 +87,22 @@ struct ExactArgs {
   const uint32_t *full_ptr;
   const uint32_t *full_doc;
   const float *full_val;
-  uint32_t n_docs;
+  uint32_t n_docs, dim;
   const uint64_t *q_indptr;
   const uint16_t *q_terms;
   const float *q_vals;
   uint32_t nq;
   uint32_t k;
-  float *acc;  // gridDim.x * n_docs floats, all zero between queries
   uint32_t *ids;
   float *scores;
+  // set by exact_layout and launch_exact: documents are taken in tiles; each
+  // query's tiles may be split over several CTAs
+  uint32_t tile, tiles, splits, area, sms;
+  uint32_t *claim, *bounds;  // [dim]: bounds of the term are done or being done; [dim][tiles + 1]
+  unsigned long long *part;  // [nq * splits][k]: the splits' results
 };
-int launch_exact(const ExactArgs &a, uint32_t grid, cudaStream_t st);
+size_t exact_layout(ExactArgs &a, uint32_t sms, void *base);  // working memory in bytes, pointers into base
+int launch_exact(ExactArgs a, cudaStream_t st);
 constexpr uint32_t kExactMaxK = 1024;
 
 // MLP and features

@@ -205,7 +205,7 @@ struct seismic_index {
   // the default search workspace (grown on demand); concurrent searches on
   // other streams bring their own
   seismic::Workspace ws;
-  seismic::DevBuf ws_exact;  // exact-search accumulators
+  seismic::DevBuf ws_exact;  // exact search: list bounds per tile, partial results
 };
 
 namespace seismic {
