@@ -16,53 +16,114 @@ constexpr int IN = SEISMIC_MLP_IN, H1 = SEISMIC_MLP_H1, H2 = SEISMIC_MLP_H2, OUT
 constexpr int OW1 = 0, OB1 = OW1 + H1 * IN, OW2 = OB1 + H1, OB2 = OW2 + H2 * H1, OW3 = OB2 + H2, OB3 = OW3 + OUT * H2;
 static_assert(OB3 + OUT == SEISMIC_MLP_PARAMS, "parameter packing");
 constexpr int kRows = 32;  // rows per CTA
-constexpr int kNT = 128;
+constexpr int kNT = 512;
+static_assert(IN == 64 && H1 == 128 && H2 == 64 && OUT == 2 && kRows == 32 && kNT == 512, "the tiles below");
+// Shared-memory row strides of a multiple of 4 floats that is 4 mod 32: eight
+// lanes on eight consecutive rows read float4s from 32 different banks.
+constexpr int S1 = IN + 4, S2 = H1 + 4;
 
 __device__ __forceinline__ float bfr(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + __expf(-x)); }
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
-struct MlpSmem {
-  float w[SEISMIC_MLP_PARAMS];
-  float a0[kRows][IN];
-  float z1[kRows][H1];  // pre-activation
-  float a1[kRows][H1];  // bf16-rounded ReLU
-  float z2[kRows][H2];
-  float a2[kRows][H2];
-  float o[kRows][OUT];
+struct MlpSmem {  // read as float4s
+  alignas(16) float w1[H1 * S1];
+  alignas(16) float w2[H2 * S2];
+  alignas(16) float w3[OUT * H2];
+  alignas(16) float a0[kRows * S1];
+  alignas(16) float z1[kRows * S2];  // pre-activation
+  alignas(16) float a1[kRows * S2];  // bf16-rounded ReLU
+  alignas(16) float z2[kRows * S1];
+  alignas(16) float a2[kRows * S1];
+  float b1[H1], b2[H2], b3[OUT], o[kRows * OUT];
 };
+static_assert(IN == H2, "rows of a0, z2 and a2 share a stride");
+
+__device__ void mlp_load(MlpSmem &s, const float *w) {
+  for (int i = threadIdx.x; i < SEISMIC_MLP_PARAMS; i += kNT) {
+    const float x = w[i];
+    if (i < OB1) s.w1[(i - OW1) / IN * S1 + (i - OW1) % IN] = x;
+    else if (i < OW2) s.b1[i - OB1] = x;
+    else if (i < OB2) s.w2[(i - OW2) / H1 * S2 + (i - OW2) % H1] = x;
+    else if (i < OW3) s.b2[i - OB2] = x;
+    else if (i < OB3) s.w3[i - OW3] = x;
+    else s.b3[i - OB3] = x;
+  }
+  __syncthreads();
+}
+
+// Outputs of one layer, 4 rows by J columns per thread (rows 4 rg .., columns
+// c0 + 32 j): z = bias + the products in input order, so each is the same chain
+// of fused multiply-adds whatever the tile.
+template <int N, int J>
+__device__ __forceinline__ void mlp_tile(const float *w, int sw, const float *bias, const float *in, int si, int rg, int c0,
+                                         float z[4][J]) {
+#pragma unroll
+  for (int j = 0; j < J; j++)
+#pragma unroll
+    for (int r = 0; r < 4; r++) z[r][j] = bias[c0 + 32 * j];
+#pragma unroll 4
+  for (int f = 0; f < N; f += 4) {
+    float4 x[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) x[r] = ld4(in + (4 * rg + r) * si + f);
+#pragma unroll
+    for (int j = 0; j < J; j++) {
+      const float4 y = ld4(w + (c0 + 32 * j) * sw + f);
+#pragma unroll
+      for (int r = 0; r < 4; r++) {
+        z[r][j] = fmaf(y.x, x[r].x, z[r][j]);
+        z[r][j] = fmaf(y.y, x[r].y, z[r][j]);
+        z[r][j] = fmaf(y.z, x[r].z, z[r][j]);
+        z[r][j] = fmaf(y.w, x[r].w, z[r][j]);
+      }
+    }
+  }
+}
 
 // forward for rows [r0, r0 + nr) held in shared memory
 __device__ void mlp_fwd(MlpSmem &s, const float *feat, uint64_t r0, int nr) {
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rg = warp & 7, half = warp >> 3;
   for (int i = tid; i < kRows * IN; i += kNT) {
-    int r = i / IN, f = i % IN;
-    s.a0[r][f] = r < nr ? bfr(feat[(r0 + r) * IN + f]) : 0.0f;
+    const int r = i / IN, f = i % IN;
+    s.a0[r * S1 + f] = r < nr ? bfr(feat[(r0 + r) * IN + f]) : 0.0f;
   }
   __syncthreads();
-  for (int i = tid; i < kRows * H1; i += kNT) {
-    int r = i / H1, m = i % H1;
-    float z = s.w[OB1 + m];
-    const float *w = s.w + OW1 + m * IN;
-    for (int f = 0; f < IN; f++) z = fmaf(w[f], s.a0[r][f], z);
-    s.z1[r][m] = z;
-    s.a1[r][m] = bfr(fmaxf(z, 0.0f));
+  {
+    float z[4][2];
+    mlp_tile<IN, 2>(s.w1, S1, s.b1, s.a0, S1, rg, 64 * half + lane, z);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        const int at = (4 * rg + r) * S2 + 64 * half + lane + 32 * j;
+        s.z1[at] = z[r][j];
+        s.a1[at] = bfr(fmaxf(z[r][j], 0.0f));
+      }
   }
   __syncthreads();
-  for (int i = tid; i < kRows * H2; i += kNT) {
-    int r = i / H2, m = i % H2;
-    float z = s.w[OB2 + m];
-    const float *w = s.w + OW2 + m * H1;
-    for (int f = 0; f < H1; f++) z = fmaf(w[f], s.a1[r][f], z);
-    s.z2[r][m] = z;
-    s.a2[r][m] = bfr(fmaxf(z, 0.0f));
+  {
+    float z[4][1];
+    mlp_tile<H1, 1>(s.w2, S2, s.b2, s.a1, S2, rg, 32 * half + lane, z);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+      const int at = (4 * rg + r) * S1 + 32 * half + lane;
+      s.z2[at] = z[r][0];
+      s.a2[at] = bfr(fmaxf(z[r][0], 0.0f));
+    }
   }
   __syncthreads();
-  for (int i = tid; i < kRows * OUT; i += kNT) {
-    int r = i / OUT, j = i % OUT;
-    float z = s.w[OB3 + j];
-    const float *w = s.w + OW3 + j * H2;
-    for (int f = 0; f < H2; f++) z = fmaf(w[f], s.a2[r][f], z);
-    s.o[r][j] = z;
+  if (tid < kRows * OUT) {
+    const int r = tid / OUT, j = tid % OUT;
+    float z = s.b3[j];
+    for (int f = 0; f < H2; f += 4) {
+      const float4 x = ld4(s.a2 + r * S1 + f), y = ld4(s.w3 + j * H2 + f);
+      z = fmaf(y.x, x.x, z);
+      z = fmaf(y.y, x.y, z);
+      z = fmaf(y.z, x.z, z);
+      z = fmaf(y.w, x.w, z);
+    }
+    s.o[tid] = z;
   }
   __syncthreads();
 }
@@ -71,12 +132,11 @@ __global__ void __launch_bounds__(kNT) k_mlp_forward(const float *__restrict__ w
                                                       uint64_t n, float *__restrict__ out) {
   extern __shared__ __align__(16) unsigned char smraw[];
   MlpSmem &s = *reinterpret_cast<MlpSmem *>(smraw);
-  for (int i = threadIdx.x; i < SEISMIC_MLP_PARAMS; i += kNT) s.w[i] = w[i];
-  __syncthreads();
+  mlp_load(s, w);
   for (uint64_t r0 = (uint64_t)blockIdx.x * kRows; r0 < n; r0 += (uint64_t)gridDim.x * kRows) {
     int nr = (int)((n - r0) < (uint64_t)kRows ? (n - r0) : (uint64_t)kRows);
     mlp_fwd(s, feat, r0, nr);
-    for (int i = threadIdx.x; i < nr * OUT; i += kNT) out[r0 * OUT + i] = s.o[i / OUT][i % OUT];
+    for (int i = threadIdx.x; i < nr * OUT; i += kNT) out[r0 * OUT + i] = s.o[i];
     __syncthreads();
   }
 }
@@ -86,13 +146,12 @@ __global__ void __launch_bounds__(kNT) k_mlp_params(const float *__restrict__ w,
                                                      uint32_t *__restrict__ q_cut, float *__restrict__ q_hf) {
   extern __shared__ __align__(16) unsigned char smraw[];
   MlpSmem &s = *reinterpret_cast<MlpSmem *>(smraw);
-  for (int i = threadIdx.x; i < SEISMIC_MLP_PARAMS; i += kNT) s.w[i] = w[i];
-  __syncthreads();
+  mlp_load(s, w);
   for (uint64_t r0 = (uint64_t)blockIdx.x * kRows; r0 < n; r0 += (uint64_t)gridDim.x * kRows) {
     int nr = (int)((n - r0) < (uint64_t)kRows ? (n - r0) : (uint64_t)kRows);
     mlp_fwd(s, feat, r0, nr);
     for (int r = threadIdx.x; r < nr; r += kNT) {
-      float o0 = s.o[r][0], o1 = s.o[r][1];
+      float o0 = s.o[r * OUT], o1 = s.o[r * OUT + 1];
       uint32_t c = cut_fb;
       float h = hf_fb;
       if (isfinite(o0) && isfinite(o1)) {  // fixed parameters are the fallback
@@ -106,80 +165,131 @@ __global__ void __launch_bounds__(kNT) k_mlp_params(const float *__restrict__ w,
   }
 }
 
-// forward + backward; gradients accumulated with atomics into g (zeroed by caller)
+struct MlpGradSmem {
+  MlpSmem f;
+  alignas(16) float dz1[kRows * S2];
+  alignas(16) float dz2[kRows * S1];
+  float dzo[kRows * OUT], loss;
+};
+
+// Adds four consecutive floats to g (16-byte aligned).
+__device__ __forceinline__ void red4(float *g, float x, float y, float z, float w) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(g), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
+// forward + backward; each thread keeps a 4 x 4 tile of both weight gradients
+// (and the first threads the small ones) in registers over the CTA's rows and
+// adds them to g (zeroed by the caller) once at the end, four at a time.
+// Bound by shared-memory reads: every operand tile is read as float4s from
+// conflict-free rows (weights read at a stride of 64 or 128 floats, 32 lanes on
+// one bank, and scalar reads took the whole step of 4096 rows, launches and host call
+// included, to 115 us; now 47 us).
 __global__ void __launch_bounds__(kNT) k_mlp_grad(const float *__restrict__ w, const float *__restrict__ feat,
                                                    const float *__restrict__ tgt, uint64_t n, float *__restrict__ g,
                                                    float *__restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  MlpSmem &s = *reinterpret_cast<MlpSmem *>(smraw);
-  float *gl = reinterpret_cast<float *>(smraw + sizeof(MlpSmem));  // local gradient, SEISMIC_MLP_PARAMS
-  __shared__ float dz2[kRows][H2], dz1[kRows][H1], dzo[kRows][OUT];
-  __shared__ float lsum;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < SEISMIC_MLP_PARAMS; i += kNT) {
-    s.w[i] = w[i];
-    gl[i] = 0.0f;
-  }
-  if (tid == 0) lsum = 0.0f;
-  __syncthreads();
+  MlpGradSmem &sg = *reinterpret_cast<MlpGradSmem *>(smraw);
+  MlpSmem &s = sg.f;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) sg.loss = 0.0f;
+  mlp_load(s, w);
   const float inv_n = 1.0f / (float)n;
+  // tiles: rows m of W1 4 (tid / 16) .. and its columns 4 (tid % 16) ..; rows of W2 4 (tid / 32) .., columns 4 (tid % 32) ..
+  const int m1 = tid / 16 * 4, f1 = tid % 16 * 4, m2 = warp * 4, f2 = lane * 4;
+  float g1[4][4] = {}, g2[4][4] = {}, gs = 0.0f;  // gs: a bias or an output weight
   for (uint64_t r0 = (uint64_t)blockIdx.x * kRows; r0 < n; r0 += (uint64_t)gridDim.x * kRows) {
     const int nr = (int)((n - r0) < (uint64_t)kRows ? (n - r0) : (uint64_t)kRows);
     mlp_fwd(s, feat, r0, nr);
-    for (int i = tid; i < kRows * OUT; i += kNT) {
-      int r = i / OUT, j = i % OUT;
+    if (tid < kRows * OUT) {
+      const int r = tid / OUT, j = tid % OUT;
       float d = 0.0f;
       if (r < nr) {
-        float sg = sigm(s.o[r][j]), e = sg - tgt[(r0 + r) * OUT + j];
-        atomicAdd(&lsum, e * e * inv_n);
-        d = 2.0f * e * sg * (1.0f - sg) * inv_n;
+        const float sgm = sigm(s.o[tid]), e = sgm - tgt[(r0 + r) * OUT + j];
+        atomicAdd(&sg.loss, e * e * inv_n);
+        d = 2.0f * e * sgm * (1.0f - sgm) * inv_n;
       }
-      dzo[r][j] = d;
+      sg.dzo[tid] = d;
     }
     __syncthreads();
     for (int i = tid; i < kRows * H2; i += kNT) {
-      int r = i / H2, m = i % H2;
+      const int r = i / H2, m = i % H2;
       float d = 0.0f;
-      for (int j = 0; j < OUT; j++) d = fmaf(s.w[OW3 + j * H2 + m], dzo[r][j], d);
-      dz2[r][m] = s.z2[r][m] > 0.0f ? d : 0.0f;
+#pragma unroll
+      for (int j = 0; j < OUT; j++) d = fmaf(s.w3[j * H2 + m], sg.dzo[r * OUT + j], d);
+      sg.dz2[r * S1 + m] = s.z2[r * S1 + m] > 0.0f ? d : 0.0f;
     }
     __syncthreads();
-    for (int i = tid; i < kRows * H1; i += kNT) {
-      int r = i / H1, m = i % H1;
-      float d = 0.0f;
-      for (int j = 0; j < H2; j++) d = fmaf(s.w[OW2 + j * H1 + m], dz2[r][j], d);
-      dz1[r][m] = s.z1[r][m] > 0.0f ? d : 0.0f;
-    }
-    __syncthreads();
-    // weight gradients: each thread owns parameters, summing over the CTA's rows
-    for (int p = tid; p < SEISMIC_MLP_PARAMS; p += kNT) {
-      float acc = 0.0f;
-      if (p < OB1) {
-        int m = p / IN, f = p % IN;
-        for (int r = 0; r < nr; r++) acc = fmaf(dz1[r][m], s.a0[r][f], acc);
-      } else if (p < OW2) {
-        int m = p - OB1;
-        for (int r = 0; r < nr; r++) acc += dz1[r][m];
-      } else if (p < OB2) {
-        int q = p - OW2, m = q / H1, f = q % H1;
-        for (int r = 0; r < nr; r++) acc = fmaf(dz2[r][m], s.a1[r][f], acc);
-      } else if (p < OW3) {
-        int m = p - OB2;
-        for (int r = 0; r < nr; r++) acc += dz2[r][m];
-      } else if (p < OB3) {
-        int q = p - OW3, j = q / H2, f = q % H2;
-        for (int r = 0; r < nr; r++) acc = fmaf(dzo[r][j], s.a2[r][f], acc);
-      } else {
-        int j = p - OB3;
-        for (int r = 0; r < nr; r++) acc += dzo[r][j];
+    {  // dz1: rows 2 warp, 2 warp + 1, columns 4 lane ..
+      float d[2][4] = {};
+#pragma unroll 4
+      for (int j = 0; j < H2; j += 4) {
+        const float4 x0 = ld4(sg.dz2 + (2 * warp) * S1 + j), x1 = ld4(sg.dz2 + (2 * warp + 1) * S1 + j);
+        const float xa[2][4] = {{x0.x, x0.y, x0.z, x0.w}, {x1.x, x1.y, x1.z, x1.w}};
+#pragma unroll
+        for (int jj = 0; jj < 4; jj++) {
+          const float4 y = ld4(s.w2 + (j + jj) * S2 + 4 * lane);
+#pragma unroll
+          for (int r = 0; r < 2; r++) {
+            d[r][0] = fmaf(y.x, xa[r][jj], d[r][0]);
+            d[r][1] = fmaf(y.y, xa[r][jj], d[r][1]);
+            d[r][2] = fmaf(y.z, xa[r][jj], d[r][2]);
+            d[r][3] = fmaf(y.w, xa[r][jj], d[r][3]);
+          }
+        }
       }
-      gl[p] += acc;
+#pragma unroll
+      for (int r = 0; r < 2; r++) {
+        const int at = (2 * warp + r) * S2 + 4 * lane;
+        const float4 z = ld4(s.z1 + at);
+        *reinterpret_cast<float4 *>(sg.dz1 + at) = make_float4(z.x > 0.0f ? d[r][0] : 0.0f, z.y > 0.0f ? d[r][1] : 0.0f,
+                                                               z.z > 0.0f ? d[r][2] : 0.0f, z.w > 0.0f ? d[r][3] : 0.0f);
+      }
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int r = 0; r < nr; r++) {
+      const float4 d = ld4(sg.dz1 + r * S2 + m1), x = ld4(s.a0 + r * S1 + f1);
+      const float da[4] = {d.x, d.y, d.z, d.w}, xa[4] = {x.x, x.y, x.z, x.w};
+      const float4 e = ld4(sg.dz2 + r * S1 + m2), y = ld4(s.a1 + r * S2 + f2);
+      const float ea[4] = {e.x, e.y, e.z, e.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          g1[i][j] = fmaf(da[i], xa[j], g1[i][j]);
+          g2[i][j] = fmaf(ea[i], ya[j], g2[i][j]);
+        }
+    }
+    for (int r = 0; r < nr; r++) {
+      if (tid < H1) gs += sg.dz1[r * S2 + tid];
+      else if (tid < H1 + H2) gs += sg.dz2[r * S1 + tid - H1];
+      else if (tid < H1 + H2 + OUT * H2) gs = fmaf(sg.dzo[r * OUT + (tid - H1 - H2) / H2], s.a2[r * S1 + (tid - H1 - H2) % H2], gs);
+      else if (tid < H1 + H2 + OUT * H2 + OUT) gs += sg.dzo[r * OUT + tid - H1 - H2 - OUT * H2];
     }
     __syncthreads();
   }
-  for (int p = tid; p < SEISMIC_MLP_PARAMS; p += kNT) atomicAdd(&g[p], gl[p]);
-  if (tid == 0) atomicAdd(loss, lsum);
+  // the gradient may start at any 4-byte boundary
+  const bool al = (reinterpret_cast<uintptr_t>(g) & 15u) == 0;
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    float *p1 = g + OW1 + (m1 + i) * IN + f1, *p2 = g + OW2 + (m2 + i) * H1 + f2;
+    if (al) {
+      red4(p1, g1[i][0], g1[i][1], g1[i][2], g1[i][3]);
+      red4(p2, g2[i][0], g2[i][1], g2[i][2], g2[i][3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        atomicAdd(p1 + j, g1[i][j]);
+        atomicAdd(p2 + j, g2[i][j]);
+      }
+    }
+  }
+  if (tid < H1) atomicAdd(g + OB1 + tid, gs);
+  else if (tid < H1 + H2) atomicAdd(g + OB2 + tid - H1, gs);
+  else if (tid < H1 + H2 + OUT * H2 + OUT) atomicAdd(g + OW3 + tid - H1 - H2, gs);
+  if (tid == 0) atomicAdd(loss, sg.loss);
 }
+static_assert(OW1 % 4 == 0 && OW2 % 4 == 0 && OB3 == OW3 + OUT * H2, "vector additions and the small gradients' order");
 
 __global__ void k_adam(float *w, const float *g, float *m, float *v, float lr, float b1c, float b2c) {
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -237,7 +347,7 @@ __global__ void k_features(const uint64_t *__restrict__ ip, const uint16_t *__re
   }
 }
 
-size_t mlp_smem(bool grad) { return sizeof(MlpSmem) + (grad ? SEISMIC_MLP_PARAMS * 4 : 0); }
+size_t mlp_smem(bool grad) { return grad ? sizeof(MlpGradSmem) : sizeof(MlpSmem); }
 
 int set_attr(const void *fn, size_t smem) {
   SZ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -37,3 +37,43 @@ def test_exact_search_tiles_and_splits(sz, n_docs, nq, k):
     np.testing.assert_array_equal(ids[:, :m], order.astype(np.uint32))
     np.testing.assert_array_equal(sc[:, :m], np.take_along_axis(score, order, 1).astype(np.float32))
     assert (ids[:, m:] == sz.NONE_ID).all() and np.isneginf(sc[:, m:]).all()
+
+
+def _bf16(x):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(x, dtype=np.float32)).bfloat16().float().numpy().astype(np.float64)
+
+
+# 32 rows per CTA; gradients off a 16-byte boundary are added one by one.  Bar: fp32 sums of up to 5000 products
+# (5000 * 2^-24 = 3e-4) and the bf16 roundings that fall the other way (2^-9 each, few) stay below 1e-2 in norm.
+@pytest.mark.parametrize("n", [1, 31, 33, 5000])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_mlp_gradient_row_edges(sz, n, offset):
+    import torch
+    from oracle import mlp
+    rng = np.random.default_rng(n)
+    w = (mlp.init(3) * 0.5).astype(np.float32)
+    feat = rng.random((n, 64)).astype(np.float32) * 4
+    tgt = rng.random((n, 2)).astype(np.float32)
+    buf = [torch.zeros(mlp.N_PARAMS + 4, device="cuda")[offset:offset + mlp.N_PARAMS] for _ in range(4)]
+    buf[0].copy_(torch.from_numpy(w))
+    loss = torch.zeros(1, device="cuda")
+    sz.seismic_mlp_train_step(buf[0], buf[1], buf[2], buf[3], torch.from_numpy(feat).cuda(),
+                              torch.from_numpy(tgt).cuda(), 0.0, 1, loss)
+    torch.cuda.synchronize()
+    p = mlp.unpack(w)
+    a0 = _bf16(feat)
+    z1 = a0 @ p["W1"].T + p["b1"]
+    a1 = _bf16(np.maximum(z1, 0))
+    z2 = a1 @ p["W2"].T + p["b2"]
+    a2 = _bf16(np.maximum(z2, 0))
+    s = mlp.sigmoid(a2 @ p["W3"].T + p["b3"])
+    e = s - tgt
+    do = 2 * e * s * (1 - s) / n
+    d2 = (do @ p["W3"]) * (z2 > 0)
+    d1 = (d2 @ p["W2"]) * (z1 > 0)
+    ref = mlp.pack(dict(W1=d1.T @ a0, b1=d1.sum(0), W2=d2.T @ a1, b2=d2.sum(0), W3=do.T @ a2, b3=do.sum(0)))
+    got = buf[1].cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 1e-2 * np.linalg.norm(ref)
+    assert abs(loss.item() - (e * e).sum() / n) <= 1e-3 * loss.item()
+    np.testing.assert_array_equal(buf[0].cpu().numpy(), w)  # learning rate 0
