@@ -100,25 +100,29 @@ typedef struct {
                             predictions fall back to (cut, heap_factor) above */
   uint32_t wave;         /* blocks evaluated per threshold update; 1 (default) keeps the
                             sequential visiting order of the algorithm exactly */
-  uint32_t group;        /* how documents are scored.  CTA shape: 1 = every thread of the CTA
-                            takes row chunks of the whole wave (chunk-flattened; seen documents
-                            are dropped before their rows are read), 8/16/32 = lane groups of
+  uint32_t group;        /* how documents are scored.  CTA shape: 1 = each warp goes over the rows
+                            of its share of the wave laid end to end (seen documents are dropped
+                            before their rows are read; small waves are scored together, with the
+                            results and counters of one after the other), 8/16/32 = lane groups of
                             that width score one row each.  Warp shape: 4/8/16/32 lanes per
                             row.  0 = 1 on the CTA shape, 8 on the warp shape.  Scores differ
                             only in fp32 summation order */
-  uint32_t cta_warps;    /* warps per CTA: 4, 8 or 16; 0 = 8 */
+  uint32_t cta_warps;    /* warps per CTA: 4, 8 or 16; 0 = 8, or more with group 1 and fewer queries
+                            than the GPU holds (the results are those of 8) */
   uint32_t persistent;   /* 1: one persistent launch that pulls queries from a device queue */
   uint32_t max_query_nnz; /* device queries: an upper bound on any query's nonzeros, which sizes
                             shared memory; 0 = measure it (one device synchronisation, so not
                             inside stream capture).  Ignored for host queries. */
-  uint32_t hash_slots;   /* per-query seen-set slots (power of two); 0 = 2048.  A full set only
-                            costs repeated work, never a different result */
+  uint32_t hash_slots;   /* launches that are not persistent: per-query seen-set slots (power of two);
+                            0 = 2048, or with group 1 a bitmap of a collection of up to 131,072
+                            documents.  A full set only costs repeated work, never a different
+                            result */
   uint32_t shape;        /* 0 or 1: one CTA per query (any k, any wave; the measured fastest);
                             2: one warp per query (k <= 128, wave 1, persistent, cta_warps
                             independent warps per CTA: 1/2/4, 0 = 4).  Both keep the
                             algorithm's sequential order at wave 1 */
-  int32_t no_prefetch;   /* 1 turns off the L2 bulk prefetch of upcoming member lists and rows
-                            (a speed knob; results are the same) */
+  int32_t no_prefetch;   /* 1 turns off the L2 bulk prefetch of upcoming member lists and, outside
+                            group 1, rows (a speed knob; results are the same) */
   uint32_t order;        /* persistent launches: 0 (default) runs queries grouped by their
                             largest term, so queries reading the same lists share L2; 1 runs
                             them in input order; 2 runs the queries that traverse the most

@@ -17,13 +17,14 @@
 //  H4  a block is skipped iff the top-k is full and r < hf * theta (or
 //      r < theta / hf); r is non-increasing and theta non-decreasing along
 //      the order, so the first skipped block ends the list.
-//  H5  forward rows: groups of G lanes score one document each; a row is a
-//      record of 8-entry chunks read with 16-byte vector loads.  At the start
-//      of a wave every row of the wave is prefetched into L2 with one TMA bulk
-//      prefetch per document, and the member lists of the next wave's blocks
-//      too, so the groups' sequential row reads hit L2.  Each document is
-//      scored at most once per query (a global bitmap per persistent CTA, or
-//      a bounded shared-memory hash set).
+//  H5  forward rows: each warp takes some of a wave's documents and goes over
+//      their rows laid end to end (group 1), or groups of G lanes score one
+//      document each; a row is a record of 8-entry chunks read with 16- and
+//      32-byte vector loads.  With lane groups every row of a wave is
+//      prefetched into L2 at its start, one TMA bulk prefetch per document; the
+//      member lists of the next blocks are always.  Each document is scored at
+//      most once per query (a global bitmap per persistent CTA, a bitmap in
+//      shared memory for a small collection, or a bounded shared-memory hash set).
 //  H6  top-k by (score desc, id asc): candidates that beat the k-th score are
 //      collected per wave and merged by rank.
 //  H7  kappa-NN expansion of the top-k after the lists (S fixed first).
@@ -43,17 +44,25 @@ namespace {
 
 using namespace dev;
 
-// Insert d into the per-query seen set; true when d was not there before
-// (or the set is too crowded to tell, in which case d is scored again).
-__device__ __forceinline__ bool seen_insert(uint32_t *tab, uint32_t hs_mask, uint32_t d, uint32_t *full) {
+// Insert d into the per-query seen set; true when d was not there before (or
+// the set cannot tell, in which case d is scored again).  A set that is three
+// quarters full stops probing: a document takes its slot whatever is there, so a lookup
+// stays one atomic, and what was there is forgotten.  (Few documents are met
+// twice -- 3 % of a search of 34,000 -- so forgetting costs little, while 16 probes
+// per document made one query over 1M documents take 2.4 ms instead of 1.8.)
+__device__ __forceinline__ bool seen_insert(uint32_t *tab, uint32_t hs_mask, uint32_t d, bool crowded, uint32_t *full) {
   const uint32_t key = d + 1u;
   uint32_t h = (d * 0x9E3779B1u) & hs_mask;
+  if (!crowded) {
 #pragma unroll 1
-  for (int p = 0; p < 16; p++) {
-    uint32_t old = atomicCAS(&tab[h], 0u, key);
-    if (old == 0u) return true;
-    if (old == key) return false;
-    h = (h + 1u) & hs_mask;
+    for (int p = 0; p < 16; p++) {
+      uint32_t old = atomicCAS(&tab[h], 0u, key);
+      if (old == 0u) return true;
+      if (old == key) return false;
+      h = (h + 1u) & hs_mask;
+    }
+  } else if (atomicExch(&tab[h], key) == key) {
+    return false;
   }
   *full = 1u;
   return true;
@@ -99,9 +108,12 @@ __device__ uint32_t block_rank_scan(const uint32_t *bits, uint16_t *rank, uint32
 // when used, so no pointer to them stays live in a register.
 extern __shared__ __align__(16) unsigned char g_sm[];
 
+struct WarpDocs;
+
 struct Smem {
   const SearchArgs &a;
-  uint32_t *seen;  // this CTA's global bitmap, or NULL
+  uint32_t *seen;  // this CTA's seen bitmap (global memory, or shared for a small collection), or NULL: the hash set
+  uint32_t turn;   // the wave's candidate counter
   __device__ __forceinline__ uint32_t *qbits() const { return reinterpret_cast<uint32_t *>(g_sm + a.off_qbits); }
   __device__ __forceinline__ uint16_t *qrank() const { return reinterpret_cast<uint16_t *>(g_sm + a.off_qrank); }
   __device__ __forceinline__ float *qval() const { return reinterpret_cast<float *>(g_sm + a.off_qval); }
@@ -121,30 +133,35 @@ struct Smem {
   __device__ __forceinline__ uint32_t *cand_id() const { return reinterpret_cast<uint32_t *>(g_sm + a.off_cand_id); }
   __device__ __forceinline__ uint8_t *cand_ok() const { return reinterpret_cast<uint8_t *>(g_sm + a.off_cand_ok); }
   __device__ __forceinline__ uint32_t *bptr() const { return reinterpret_cast<uint32_t *>(g_sm + a.off_bptr); }
-  __device__ __forceinline__ uint32_t *fdoc() const { return reinterpret_cast<uint32_t *>(g_sm + a.off_fdoc); }
-  __device__ __forceinline__ uint32_t *fc0() const { return reinterpret_cast<uint32_t *>(g_sm + a.off_fc0); }
-  __device__ __forceinline__ uint32_t *fpre() const { return reinterpret_cast<uint32_t *>(g_sm + a.off_fpre); }
-  __device__ __forceinline__ uint8_t *cmap() const { return reinterpret_cast<uint8_t *>(g_sm + a.off_cmap); }
+  __device__ __forceinline__ WarpDocs *wdocs() const { return reinterpret_cast<WarpDocs *>(g_sm + a.off_wdocs); }
+  __device__ __forceinline__ unsigned char *wqueue() const { return g_sm + a.off_wqueue; }
+  __device__ __forceinline__ uint16_t *cand_i() const { return reinterpret_cast<uint16_t *>(g_sm + a.off_cand_i); }
+  __device__ __forceinline__ uint8_t *fresh() const { return reinterpret_cast<uint8_t *>(g_sm + a.off_fresh); }
+  __device__ __forceinline__ uint8_t *qfilt() const { return reinterpret_cast<uint8_t *>(g_sm + a.off_qfilt); }
 };
 
 struct Shared {
-  uint32_t q, nzq, ncut, count, ncand, nvalid, hash_full, bad;
+  uint32_t q, nzq, ncut, count, nvalid, hash_full, hash_n, bad;
+  uint32_t ncand[2];  // candidates of a wave; waves take turns, so one may begin while another's count is still read
   float hf;
   uint32_t cut;
   uint32_t wtmp[32];
   unsigned long long st[SEISMIC_STATS_N];
 };
 
-// The members of the wave's blocks keys[0 .. nw) (sorted positions) of the
-// current list, as one run: member i is found by walking the blocks' sizes in
-// shared memory, so forming a wave needs no barrier.
-struct WaveBlocks {
+// Members of the current list: of the blocks keys[0 .. nw) (sorted positions),
+// as one run -- member i is found by walking the blocks' sizes in shared memory,
+// so forming a wave needs no barrier -- or, with nw = 0, the list's own order.
+// Either way starting with member i0.
+struct ListSrc {
   const unsigned long long *keys;
   const uint32_t *bptr;
-  uint32_t nw;
+  uint32_t nw, i0;
   const uint32_t *ids;
   const unsigned long long *rows;
   __device__ __forceinline__ uint32_t at(uint32_t i) const {
+    i += i0;
+    if (nw == 0) return i;
     uint32_t b = (uint32_t)(keys[0] & 0xFFFFFFFFu), lo = bptr[b], nd = bptr[b + 1] - lo;
     for (uint32_t w = 1; w < nw && i >= nd; w++) {
       i -= nd;
@@ -154,8 +171,6 @@ struct WaveBlocks {
     }
     return lo + i;
   }
-  __device__ __forceinline__ uint32_t id(uint32_t i) const { return __ldg(ids + at(i)); }
-  __device__ __forceinline__ unsigned long long row(uint32_t i, uint32_t) const { return __ldg(rows + at(i)); }
   __device__ __forceinline__ void fetch(uint32_t i, uint32_t &d, unsigned long long &r) const {
     const uint32_t m = at(i);
     d = __ldg(ids + m);
@@ -163,26 +178,45 @@ struct WaveBlocks {
   }
 };
 
+// Documents by the graph: a seed document and its neighbours (ids = NULL), or
+// the neighbours of the documents ids[..], starting with the i0-th.
+struct NeighbourSrc {
+  const uint32_t *ids, *knn;
+  const unsigned long long *frow;
+  uint32_t doc, kappa, bits, i0;
+  __device__ __forceinline__ void fetch(uint32_t i, uint32_t &d, unsigned long long &r) const {
+    i += i0;
+    if (ids) d = knn_entry(knn, bits, (uint64_t)ids[i / kappa] * kappa + (i % kappa));
+    else d = i == 0 ? doc : knn_entry(knn, bits, (uint64_t)doc * kappa + (i - 1));
+    r = d == SEISMIC_NONE_ID ? 0ull : __ldg(frow + d);
+  }
+};
+
+// Ranks m candidates -- with `part`, those of the wave's members from .. to --
+// among the cnt entries of the top-k, into tmp; returns the new count.  Ends
+// with a barrier; sh.nvalid is used and has to be 0 (merge_commit clears it).
 template <int NT>
-__device__ void merge_candidates(const SearchArgs &a, Smem &s, Shared &sh) {
+__device__ uint32_t merge_rank(const SearchArgs &a, Smem &s, Shared &sh, uint32_t m, bool part, uint32_t from,
+                               uint32_t to) {
   const int tid = threadIdx.x;
-  const uint32_t m = sh.ncand, cnt = sh.count, k = a.k;
-  if (m == 0) return;  // uniform: every thread read the same ncand after the barrier
+  const uint32_t cnt = sh.count, k = a.k;
   // With the global seen bitmap a document becomes fresh once per query, so no
   // candidate repeats a heap entry or another candidate.  The bounded hash set
   // may score a document again when it is crowded: there repeats are dropped.
-  const bool check = s.seen == nullptr;
+  const bool repeats = s.seen == nullptr, check = repeats || part;
   uint32_t nvalid = m;
   if (check) {
-    const bool dupcheck = sh.hash_full != 0u;
+    const bool dupcheck = repeats && sh.hash_full != 0u;
+    auto in = [&](uint32_t i) { return !part || (s.cand_i()[i] >= from && s.cand_i()[i] < to); };
     for (uint32_t i = tid; i < m; i += NT) {
       const uint32_t id = s.cand_id()[i];
-      uint8_t ok = 1;
-      for (uint32_t j = 0; j < cnt; j++)
-        if (s.tk_id()[j] == id) { ok = 0; break; }
+      uint8_t ok = in(i) ? 1 : 0;
+      if (ok && repeats)
+        for (uint32_t j = 0; j < cnt; j++)
+          if (s.tk_id()[j] == id) { ok = 0; break; }
       if (ok && dupcheck)
         for (uint32_t j = 0; j < i; j++)
-          if (s.cand_id()[j] == id) { ok = 0; break; }
+          if (s.cand_id()[j] == id && in(j)) { ok = 0; break; }
       s.cand_ok()[i] = ok;
       if (ok) atomicAdd(&sh.nvalid, 1u);
     }
@@ -212,14 +246,23 @@ __device__ void merge_candidates(const SearchArgs &a, Smem &s, Shared &sh) {
     if (r < k) { s.tmp_s()[r] = sc; s.tmp_id()[r] = id; }
   }
   __syncthreads();
-  // nc comes from registers, so thread 0 may reset the counters in this phase
-  const uint32_t nc = min(k, cnt + nvalid);
+  return min(k, cnt + nvalid);
+}
+
+// Makes the nc ranked entries the top-k; `done` also drops the wave's candidates.
+template <int NT>
+__device__ void merge_commit(Smem &s, Shared &sh, uint32_t nc, bool done) {
+  const int tid = threadIdx.x;
   for (uint32_t i = tid; i < nc; i += NT) { s.tk_s()[i] = s.tmp_s()[i]; s.tk_id()[i] = s.tmp_id()[i]; }
-  if (tid == 0) { sh.count = nc; sh.ncand = 0; sh.nvalid = 0; }
+  if (tid == 0) {
+    sh.count = nc;
+    sh.nvalid = 0;
+    if (done) sh.ncand[s.turn ^ 1u] = 0;
+  }
   __syncthreads();
 }
 
-// Scores up to CAND documents of a source, then merges the candidates.
+// Scores up to CAND documents of a source; ends with a barrier.
 template <int G, int NT, class Src>
 __device__ void eval_wave(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, const Src &src, int knn_stage) {
   constexpr int NG = NT / G;
@@ -240,6 +283,7 @@ __device__ void eval_wave(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, 
   // Software pipeline per lane group: the next document's (id, row) are loaded
   // while the current one is scored, and the seen-bitmap test is issued with
   // the row's loads and read after the dot (a seen document's score is dropped).
+  const bool crowded = sh.hash_n > a.HS / 4 * 3;
   uint32_t dn = SEISMIC_NONE_ID;
   unsigned long long rn = 0ull;
   if ((uint32_t)grp < n) src.fetch(grp, dn, rn);
@@ -252,7 +296,7 @@ __device__ void eval_wave(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, 
     const uint32_t bit = 1u << (d & 31);
     if (gl == 0) {
       if (s.seen) old = atomicOr(s.seen + (d >> 5), bit);
-      else fresh = seen_insert(s.hash(), a.HS - 1u, d, &sh.hash_full) ? 1u : 0u;
+      else if (seen_insert(s.hash(), a.HS - 1u, d, crowded, &sh.hash_full)) { fresh = 1u; atomicAdd(&sh.hash_n, 1u); }
     }
     const float p = row_dot<G>(a.fwd_data, row, a.fp16, gl, gmask, s.qbits(), s.qrank(), s.qval());
     if (s.seen) fresh = (old & bit) ? 0u : 1u;
@@ -264,197 +308,380 @@ __device__ void eval_wave(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, 
         atomicAdd(&sh.st[knn_stage ? SEISMIC_ST_KNN_NNZ : SEISMIC_ST_DOC_NNZ], (unsigned long long)a.fwd_nnz[d]);
       }
       if (!full || better(p, d, th, thid)) {
-        uint32_t pos = atomicAdd(&sh.ncand, 1u);
+        uint32_t pos = atomicAdd(&sh.ncand[s.turn], 1u);
         s.cand_s()[pos] = p;
         s.cand_id()[pos] = d;
       }
     }
   }
   __syncthreads();
-  merge_candidates<NT>(a, s, sh);
 }
 
-// v[0..n) -> exclusive prefix sums, v[n] = the total.  Thread t takes a
-// contiguous range of ceil(n / NT) elements; warps scan their threads' sums
-// with shuffles and every thread adds the totals of the warps before it, so
-// the scan costs two barriers.  Every thread must call it (after a barrier
-// that published v).  When map is given and the total is at most cap, also
-// writes map[v[i] .. v[i+1]) = i (the owner of each unit, i < 256).
-template <int NT>
-__device__ uint32_t block_exclusive_scan(uint32_t *v, uint32_t n, uint32_t *wtmp, uint8_t *map = nullptr,
-                                         uint32_t cap = 0) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int nw = NT / 32;
-  const uint32_t per = (n + NT - 1) / NT, lo = min(n, tid * per), hi = min(n, lo + per);
-  uint32_t sum = 0;
-  for (uint32_t i = lo; i < hi; i++) sum += v[i];
-  uint32_t x = sum;
+// Which of 8 terms (two per word) may be in the query: bit e for term e.
+__device__ __forceinline__ uint32_t probe8(const uint4 &t, const uint8_t *__restrict__ filter) {
+  const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
+  uint32_t m = 0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wtmp[warp] = x;
-  __syncthreads();
-  uint32_t before = 0, total = 0;
-#pragma unroll
-  for (int w = 0; w < nw; w++) {
-    const uint32_t t = wtmp[w];
-    before += w < warp ? t : 0u;
-    total += t;
-  }
-  uint32_t run = before + x - sum;
-  const bool fill = map != nullptr && total <= cap;
-  for (uint32_t i = lo; i < hi; i++) {
-    const uint32_t c = v[i];
-    v[i] = run;
-    if (fill)
-      for (uint32_t u = 0; u < c; u++) map[run + u] = (uint8_t)i;
-    run += c;
-  }
-  if (tid == 0) v[n] = total;
-  __syncthreads();
-  return total;
+  for (int e = 0; e < 8; e++)
+    m += (uint32_t)filter[((e & 1) ? (tw[e >> 1] >> 16) : tw[e >> 1]) & (kFilter - 1u)] << e;
+  return m;
 }
 
-// Group 1: the wave's documents are deduplicated first (one thread each),
-// then their rows' chunks are laid end to end and scored by all threads of
-// the CTA, U chunks in flight per thread, each chunk's products with query
-// terms added in entry order; a document's score is the sum of its chunks'
-// partials in chunk order (deterministic, independent of the launch shape).
-// Work per thread is balanced whatever the row lengths; seen documents cost
-// no row reads.  fp32 rows: a chunk's values (one 32-byte sector) are read
-// only where a term is in the query (4-byte read-only loads; most chunks of a
-// row miss).  fp16 rows: a chunk is one sector, terms and values read together.
+// 16-bit value e (0 .. 7) of 8 in four words.
+__device__ __forceinline__ uint32_t pick8(const uint4 &t, uint32_t e) {
+  const uint32_t lo = (e & 2u) ? t.y : t.x, hi = (e & 2u) ? t.w : t.z;
+  return (((e & 4u) ? hi : lo) >> ((e & 1u) * 16u)) & 0xFFFFu;
+}
+
+__device__ __forceinline__ uint32_t pick16(const uint4 &t, const uint4 &t2, uint32_t e) {
+  return pick8(make_uint4((e & 8u) ? t2.x : t.x, (e & 8u) ? t2.y : t.y, (e & 8u) ? t2.z : t.z, (e & 8u) ? t2.w : t.w),
+               e & 7u);
+}
+
+// Queues a unit's candidates (the bits of m): document x, position pos0 + e,
+// terms t and t2.
+__device__ __forceinline__ void push_candidates(uint32_t *q, uint32_t m, const uint4 &t, const uint4 &t2, uint32_t x,
+                                                uint32_t pos0) {
+  const uint32_t base = (x << 27) | (pos0 << 16);
+  while (m) {
+    const uint32_t e = __ffs(m) - 1u;
+    m &= m - 1u;
+    *q++ = (base + (e << 16)) | pick16(t, t2, e);
+  }
+}
+
+// The warp's own arrays while it scores documents (group 1).  The queue holds,
+// in document, row order, the candidates of some documents -- document (5 bits)
+// | position in the row (11) | term (16); the second pass replaces an entry by
+// its chunk's partial score (the chunk's first entry) or 0 -- or, for fp16 rows,
+// the two partials of each unit with a hit.
+struct WarpDocs {
+  unsigned long long unit0[32];  // address of the document's first unit, less 32 bytes per unit of the documents before it
+  unsigned long long val[32];    // fp32 rows: address of its first value
+  uint32_t p0[32];               // units of the documents before it
+  uint32_t doc[32];
+  uint16_t nch[32];              // its 8-entry chunks
+  uint16_t start[32];            // its first queue entry
+  uint16_t member[32];           // its place in the wave
+};
+static_assert(sizeof(WarpDocs) == kWarpDocsBytes, "search_layout reserves it");
+
+// <q, row> of one row by a whole warp, a chunk per lane: chunk partials in
+// entry order, added in chunk order (every lane returns the sum).
+template <bool FP16>
+__device__ float warp_row(const SearchArgs &a, const Smem &s, unsigned long long row, uint32_t lane) {
+  const uint8_t *rec = row_base(a.fwd_data, row);
+  const uint32_t nch = (uint32_t)(row >> 32);
+  float p = 0.0f;
+  for (uint32_t c0 = 0; c0 < nch; c0 += 32) {
+    const uint32_t c = c0 + lane;
+    float acc = 0.0f;
+    if (c < nch) {
+      const uint4 t = ldg_na(chunk_terms(rec, c, FP16));
+      const uint8_t *vp = chunk_vals(rec, nch, c, FP16);
+      const uint32_t tw[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int e = 0; e < 8; e++) {
+        const float q = qlookup(s.qbits(), s.qrank(), s.qval(), (e & 1) ? (tw[e >> 1] >> 16) : (tw[e >> 1] & 0xFFFFu));
+        if (q != 0.0f)
+          acc = fmaf(q, FP16 ? __half2float(reinterpret_cast<const __half *>(vp)[e]) : reinterpret_cast<const float *>(vp)[e], acc);
+      }
+    }
+    for (uint32_t l = 0; l < 32; l++) p += __shfl_sync(0xffffffffu, acc, l);
+  }
+  return p;
+}
+
+// Group 1.  A wave's documents are dealt to the warps in runs of up to 32, one
+// per lane, and from there on a warp works by itself, without CTA barriers: it
+// drops the documents seen before, lays the others' rows end to end as units of
+// two 8-entry chunks (fp32 rows: 32 bytes of terms; fp16 rows: 64 bytes of terms
+// and values) and goes over them 32 units at a time, U such groups in flight.
+// Each term is tested against a byte filter of the query, which about 2.8 % of
+// them pass, three quarters of those being hits.
+//   fp32 rows: the candidates are queued, and a second pass takes the queue one
+//   candidate per lane: it looks the term up in the query and reads the value of
+//   a hit, so the value reads of 32 entries are in flight together and chunks
+//   without hits read no values.
+//   fp16 rows: the values came with the terms, so each lane adds its own unit's
+//   hits (queued and looked up as above: 16.2 ms where this takes 14.6; fp32 rows
+//   this way, a value read behind the other: 65.6 ms where the queue takes 63.5).
+// The products of a chunk are added in entry order, a document's chunk partials
+// in chunk order, so a score is deterministic and independent of the launch shape.
+//
+// What bounds it: issue slots and shared-memory probes, then latency -- not DRAM.
+// With every thread of the CTA on the wave's chunks, eight exact lookups per chunk
+// and 7 barriers per wave, 32 chunks took 259 warp instructions and 69 shared-
+// memory wavefronts, an L1 pipe at 77 %; a filter byte costs 3 instructions where
+// a bit of the query's bitmap and the predicated lookup cost 20.  1M documents,
+// 10k queries: cut 10, wave 8: 70.0 to 63.5 ms; cut 30 with the graph, wave 4: 149.5
+// to 137.8 ms.  300k documents, fp16 rows: 14.9 to 14.6 ms.  100k documents, every
+// block visited: 2.94 to 1.93 ms.  A filter of 4096 bytes (4.6 candidates per
+// document instead of 3.6): 67.6 ms; of 16,384 bytes (3 CTAs per SM): 65.9 ms.
+// Prefetching the rows into L2 no longer pays (64.3 ms) and is gone here.
 template <int NT, bool FP16, class Src>
 __device__ __forceinline__ void eval_wave_flat(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, const Src &src,
                                                int knn_stage) {
-  constexpr int U = 2;
-  const int tid = threadIdx.x;
+  constexpr int U = FP16 ? 1 : 2, NW = NT / 32;
+  constexpr uint32_t kUnit = FP16 ? 2u * kUnitBytes : kUnitBytes;  // bytes of two chunks: their terms (fp16 rows: and values)
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, below = (1u << lane) - 1u;
   const bool full = sh.count == a.k;
   const float th = full ? s.tk_s()[a.k - 1] : -INFINITY;
   const uint32_t thid = full ? s.tk_id()[a.k - 1] : 0u;
-  float *cpart = s.part();  // the block-score partials are dead while documents are scored
-  for (uint32_t i = tid; i < n; i += NT) {
-    uint32_t d;
-    unsigned long long row;
-    src.fetch(i, d, row);
-    uint32_t keep = SEISMIC_NONE_ID, nch = 0;
-    if (d != SEISMIC_NONE_ID) {
-      bool fresh;
-      if (s.seen) {
-        const uint32_t bit = 1u << (d & 31);
-        fresh = !(atomicOr(s.seen + (d >> 5), bit) & bit);
-      } else {
-        fresh = seen_insert(s.hash(), a.HS - 1u, d, &sh.hash_full);
-      }
-      if (fresh) {
-        keep = d;
-        nch = (uint32_t)(row >> 32);
-        if (a.prefetch) prefetch_row(a.fwd_data, row, a.fp16);
-        if (a.stats) {
-          atomicAdd(&sh.st[knn_stage ? SEISMIC_ST_KNN_DOCS : SEISMIC_ST_DOCS], 1ull);
-          atomicAdd(&sh.st[knn_stage ? SEISMIC_ST_KNN_NNZ : SEISMIC_ST_DOC_NNZ], (unsigned long long)a.fwd_nnz[d]);
+  uint32_t *ncand = &sh.ncand[s.turn];
+  auto offer = [&](float p, uint32_t d, uint32_t i) {
+    if (!full || better(p, d, th, thid)) {
+      const uint32_t pos = atomicAdd(ncand, 1u);
+      s.cand_s()[pos] = p;
+      s.cand_id()[pos] = d;
+      s.cand_i()[pos] = (uint16_t)i;
+    }
+  };
+  WarpDocs &wd = s.wdocs()[warp];
+  // a warp's queue holds the candidates of 24 units at least, or the partials of 192 units (fp16 rows)
+  constexpr uint32_t kQueue = kWarpQueueBytes / 4, kSums = kWarpQueueBytes / 8;
+  uint32_t *queue = reinterpret_cast<uint32_t *>(s.wqueue() + warp * kWarpQueueBytes);
+  float2 *sums = reinterpret_cast<float2 *>(queue);
+  const uint8_t *qf = s.qfilt();
+  const uint32_t dpw = min(32u, (n + NW - 1) / NW);
+  const bool crowded = sh.hash_n > a.HS / 4 * 3;
+  for (uint32_t r0 = 0; r0 < n; r0 += NW * 32) {  // one round, unless n > 32 NW
+    const uint32_t i = r0 + warp * dpw + lane;
+    uint32_t d = SEISMIC_NONE_ID, nch = 0;
+    unsigned long long row = 0ull;
+    if (lane < dpw && i < n) {
+      src.fetch(i, d, row);
+      bool fresh = false;
+      if (d != SEISMIC_NONE_ID) {
+        if (s.seen) {
+          const uint32_t bit = 1u << (d & 31);
+          fresh = !(atomicOr(s.seen + (d >> 5), bit) & bit);
+        } else {
+          fresh = seen_insert(s.hash(), a.HS - 1u, d, crowded, &sh.hash_full);
+        }
+        if (fresh) {
+          nch = (uint32_t)(row >> 32);
+          if (a.stats) {
+            atomicAdd(&sh.st[knn_stage ? SEISMIC_ST_KNN_DOCS : SEISMIC_ST_DOCS], 1ull);
+            atomicAdd(&sh.st[knn_stage ? SEISMIC_ST_KNN_NNZ : SEISMIC_ST_DOC_NNZ], (unsigned long long)a.fwd_nnz[d]);
+          }
+          if (!nch) offer(0.0f, d, i);  // an empty row
         }
       }
+      s.fresh()[i] = fresh ? 1 : 0;
+      if (!s.seen && fresh) atomicAdd(&sh.hash_n, 1u);
     }
-    s.fdoc()[i] = keep;
-    s.fc0()[i] = (uint32_t)row;
-    s.fpre()[i] = nch;
-  }
-  __syncthreads();
-  // the chunk map of a wave that fits one pass is written by the scan itself
-  const uint32_t all = block_exclusive_scan<NT>(s.fpre(), n, sh.wtmp, s.cmap(), a.CAPC);
-  const uint32_t *qb = s.qbits();
-  const uint16_t *qr = s.qrank();
-  const float *qv = s.qval();
-  uint32_t i0 = 0;
-  while (i0 < n) {
-    // a pass: the documents from i0 whose chunks fit in CAPC (one always does)
-    const uint32_t base = s.fpre()[i0];
-    uint32_t lo = i0 + 1, hi = n;
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi + 1) >> 1;
-      if (s.fpre()[mid] - base <= a.CAPC) lo = mid; else hi = mid - 1;
+    // rows beyond the queue's 11-bit positions go one at a time
+    uint32_t longs = __ballot_sync(0xffffffffu, nch > kShortChunks);
+    while (longs) {
+      const int l = __ffs(longs) - 1;
+      longs &= longs - 1u;
+      const unsigned long long r = __shfl_sync(0xffffffffu, row, l);
+      const float p = warp_row<FP16>(a, s, r, lane);
+      if ((int)lane == l) offer(p, d, i);
     }
-    const uint32_t i1 = lo, total = s.fpre()[i1] - base;
-    if (all > a.CAPC) {  // several passes: map this one
-      for (uint32_t i = i0 + tid; i < i1; i += NT) {
-        const uint32_t e = s.fpre()[i + 1] - base;
-        for (uint32_t c = s.fpre()[i] - base; c < e; c++) s.cmap()[c] = (uint8_t)i;  // i < CAND <= 256
-      }
-      __syncthreads();
-    }
-#pragma unroll 1
-    for (uint32_t j = tid; j < total; j += NT * U) {
-      // a row holds its chunks' terms (16 B each), then their values (32 B each):
-      // the terms are read first and a value only where the term is in the query
-      uint4 t[U], vh[U];
-      const float *vp[U];
+    const uint32_t nu = nch > kShortChunks ? 0u : (nch + 1u) / 2u;
+    uint32_t end = nu;
 #pragma unroll
-      for (int u = 0; u < U; u++) {  // past the end: the last chunk again (unconditional loads stay in registers)
-        const uint32_t jj = min(j + u * NT, total - 1u);
-        {
-          const uint32_t i = s.cmap()[jj], p0 = s.fpre()[i];
-          const uint32_t nch = s.fpre()[i + 1] - p0, o = base + jj - p0;
-          const uint8_t *rec = a.fwd_data + (size_t)s.fc0()[i] * kUnitBytes;
-          vp[u] = reinterpret_cast<const float *>(chunk_vals(rec, nch, o, FP16));
-          if (FP16) {
-            ldg_na_v8(chunk_terms(rec, o, true), t[u], vh[u]);  // the chunk's sector: terms, then halves
-          } else {
-            t[u] = ldg_na(chunk_terms(rec, o, false));
-          }
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += y;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, end, 31);
+    if (total == 0) continue;  // uniform over the warp
+    const uint32_t kept = __ballot_sync(0xffffffffu, nu != 0u), nd = __popc(kept);
+    if (nu) {
+      const uint32_t x = __popc(kept & below), p0 = end - nu;
+      const unsigned long long rec = reinterpret_cast<unsigned long long>(row_base(a.fwd_data, row));
+      wd.unit0[x] = rec - (unsigned long long)kUnit * p0;
+      if (!FP16) wd.val[x] = rec + (unsigned long long)kUnitBytes * nu;
+      wd.p0[x] = p0;
+      wd.doc[x] = d;
+      wd.nch[x] = (uint16_t)nch;
+      wd.member[x] = (uint16_t)i;
+    }
+    __syncwarp();
+    // from here on lane x stands for document x of the nd kept ones
+    const uint32_t myp0 = lane < nd ? wd.p0[lane] : total;
+    float p = 0.0f;
+    uint32_t nq = 0, wbeg = 0;  // queue entries, and the first unit they may come from
+
+    // Scores the queue's entries, which come from the units wbeg .. wend.
+    auto flush = [&](uint32_t wend) {
+      __syncwarp();
+      for (uint32_t r = 0; !FP16 && r < nq;) {
+        uint32_t cnt = min(32u, nq - r);
+        const uint32_t ent = lane < cnt ? queue[r + lane] : 0u, key = ent >> 19;  // document, chunk
+        const uint32_t prev = __shfl_up_sync(0xffffffffu, key, 1);
+        const bool first = lane == 0 || key != prev;
+        uint32_t firsts = __ballot_sync(0xffffffffu, first && lane < cnt);
+        if (r + cnt < nq && (queue[r + cnt] >> 19) == __shfl_sync(0xffffffffu, key, 31)) {
+          cnt = 31u - __clz(firsts);  // the last chunk's entries go on: it waits for the next 32 (a chunk has at most 8)
+          firsts &= (1u << cnt) - 1u;
+        }
+        const uint32_t t = ent & 0xFFFFu, w = s.qbits()[t >> 5], bit = 1u << (t & 31u);
+        const uint32_t x = ent >> 27, pos = (ent >> 16) & 0x7FFu;
+        // a row of an odd number of chunks ends in half a unit that is not its own
+        const bool hit = lane < cnt && (w & bit) && pos < 8u * wd.nch[x];
+        float q = 0.0f, v = 0.0f;
+        if (hit) {
+          q = s.qval()[s.qrank()[t >> 5] + __popc(w & (bit - 1u))];
+          v = ldg_na_f32(wd.val[x] + 4u * pos);
+        }
+        const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+        const uint32_t later = lane < 31u ? firsts & (~0u << (lane + 1u)) : 0u;
+        const uint32_t len = (firsts >> lane) & 1u ? (later ? __ffs(later) - 1u : cnt) - lane : 0u;  // a first entry's chunk
+        const uint32_t longest = __reduce_max_sync(0xffffffffu, len);
+        float acc = hit ? fmaf(q, v, 0.0f) : 0.0f;
+        for (uint32_t o = 1; o < longest; o++) {
+          const float q2 = __shfl_down_sync(0xffffffffu, q, o), v2 = __shfl_down_sync(0xffffffffu, v, o);
+          if (o < len && ((hits >> (lane + o)) & 1u)) acc = fmaf(q2, v2, acc);
+        }
+        if (lane < cnt) queue[r + lane] = len ? __float_as_uint(acc) : 0u;
+        r += cnt;
+      }
+      __syncwarp();
+      const uint32_t from = myp0 < wbeg ? 0u : myp0 < wend ? wd.start[lane] : nq;
+      uint32_t to = __shfl_down_sync(0xffffffffu, from, 1);
+      if (lane == 31) to = nq;
+      for (uint32_t e = from; e < to; e++) {
+        if constexpr (FP16) {
+          const float2 x = sums[e];
+          p += x.x;
+          p += x.y;
+        } else {
+          p += __uint_as_float(queue[e]);
+        }
+      }
+      __syncwarp();
+    };
+
+#pragma unroll 1
+    for (uint32_t j0 = 0; j0 < total; j0 += 32 * U) {
+      uint4 t[U], t2[U], h[U], h2[U];  // the two chunks' terms, fp16 rows: and values
+      uint32_t head[U], dx[U];
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        // group of units gb .. gb + 31 (past the end: the last one again, and the last unit in lanes past the
+        // end); its first unit's document, and a bit for each document that starts in it
+        const uint32_t gb = min(j0 + 32u * u, (total - 1u) & ~31u), jj = min(gb + lane, total - 1u);
+        const uint32_t x0 = __popc(__ballot_sync(0xffffffffu, myp0 <= gb)) - 1u;
+        head[u] = __reduce_or_sync(0xffffffffu, lane < nd && (myp0 & ~31u) == gb ? 1u << (myp0 & 31u) : 0u);
+        dx[u] = x0 + __popc(head[u] & ((2u << (jj & 31u)) - 2u));
+        const unsigned long long tp = wd.unit0[dx[u]] + (unsigned long long)kUnit * jj;
+        if (FP16) {  // an odd row's last unit reads 32 bytes behind the row; its candidates are dropped below
+          ldg_na_v8(reinterpret_cast<const void *>(tp), t[u], h[u]);
+          ldg_na_v8(reinterpret_cast<const void *>(tp + kUnitBytes), t2[u], h2[u]);
+        } else {
+          ldg_na_v8(reinterpret_cast<const void *>(tp), t[u], t2[u]);
         }
       }
 #pragma unroll
       for (int u = 0; u < U; u++) {
-        const uint32_t jj = j + u * NT;
-        if (jj < total) {
-          const uint32_t tw[4] = {t[u].x, t[u].y, t[u].z, t[u].w};
-          const uint32_t hw[4] = {vh[u].x, vh[u].y, vh[u].z, vh[u].w};
-          float acc = 0.0f;
-#pragma unroll
-          for (int e = 0; e < 8; e++) {  // absent terms (most) cost one shared load and no value read
-            const uint32_t tt = (e & 1) ? (tw[e >> 1] >> 16) : (tw[e >> 1] & 0xFFFFu);
-            const uint32_t w = qb[tt >> 5], sh5 = tt & 31u;
-            if ((w >> sh5) & 1u) {
-              float v;
-              if (FP16) v = __half2float(__ushort_as_half((unsigned short)((e & 1) ? (hw[e >> 1] >> 16) : (hw[e >> 1] & 0xFFFFu))));
-              else v = __ldg(vp[u] + e);
-              acc = fmaf(qv[qr[tt >> 5] + __popc(w & ((1u << sh5) - 1u))], v, acc);
+        const uint32_t gb = j0 + 32u * u;
+        if (gb >= total) break;
+        uint32_t m = probe8(t[u], qf) | probe8(t2[u], qf) << 8;
+        if (gb + lane >= total) m = 0u;
+        if constexpr (FP16) {
+          float s0 = 0.0f, s1 = 0.0f;
+          bool some = false;
+          if (m) {
+            const uint32_t x = dx[u], pos0 = 16u * (gb + lane - wd.p0[x]);
+            if (pos0 + 8u >= 8u * wd.nch[x]) m &= 0xFFu;  // a row of an odd number of chunks ends in half a unit
+            while (m) {
+              const uint32_t e = __ffs(m) - 1u;
+              m &= m - 1u;
+              const uint32_t tt = pick16(t[u], t2[u], e), w = s.qbits()[tt >> 5], bit = 1u << (tt & 31u);
+              if (w & bit) {
+                const float q = s.qval()[s.qrank()[tt >> 5] + __popc(w & (bit - 1u))];
+                const float v = __half2float(__ushort_as_half((unsigned short)pick16(h[u], h2[u], e)));
+                if (e < 8u) s0 = fmaf(q, v, s0); else s1 = fmaf(q, v, s1);
+                some = true;
+              }
             }
           }
-          cpart[jj] = acc;
+          const uint32_t ball = __ballot_sync(0xffffffffu, some);
+          if (nq + __popc(ball) > kSums) {
+            flush(gb);
+            nq = 0;
+            wbeg = gb;
+          }
+          const uint32_t at = nq + __popc(ball & below);
+          if ((head[u] >> lane) & 1u) wd.start[dx[u]] = (uint16_t)at;
+          if (some) sums[at] = make_float2(s0, s1);
+          nq += __popc(ball);
+          continue;
         }
+        const uint32_t c = __popc(m);
+        uint32_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += y;
+        }
+        const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
+        if (nq + tot > kQueue) {
+          flush(gb);
+          nq = 0;
+          wbeg = gb;
+        }
+        // a group with more candidates than the queue holds goes in two halves of 16 units
+        const bool halves = tot > kQueue;
+        uint32_t at = nq + inc - c, mid = 0;
+        if (halves) {
+          mid = __shfl_sync(0xffffffffu, inc, 15);
+          if (lane >= 16) at -= mid;
+          if (lane < 16) {
+            if ((head[u] >> lane) & 1u) wd.start[dx[u]] = (uint16_t)at;
+            push_candidates(queue + at, m, t[u], t2[u], dx[u], 16u * (gb + lane - wd.p0[dx[u]]));
+          }
+          nq = mid;
+          flush(gb + 16u);
+          nq = 0;
+          wbeg = gb + 16u;
+        }
+        if (!halves || lane >= 16) {
+          if ((head[u] >> lane) & 1u) wd.start[dx[u]] = (uint16_t)at;
+          if (m) push_candidates(queue + at, m, t[u], t2[u], dx[u], 16u * (gb + lane - wd.p0[dx[u]]));
+        }
+        nq += halves ? tot - mid : tot;
       }
     }
-    __syncthreads();
-    for (uint32_t i = i0 + tid; i < i1; i += NT) {
-      const uint32_t d = s.fdoc()[i];
-      if (d == SEISMIC_NONE_ID) continue;
-      const uint32_t e = s.fpre()[i + 1] - base;
-      float p = 0.0f;
-      for (uint32_t c = s.fpre()[i] - base; c < e; c++) p += cpart[c];
-      if (!full || better(p, d, th, thid)) {
-        const uint32_t pos = atomicAdd(&sh.ncand, 1u);
-        s.cand_s()[pos] = p;
-        s.cand_id()[pos] = d;
-      }
-    }
-    __syncthreads();
-    i0 = i1;
+    flush(total);
+    if (lane < nd) offer(p, wd.doc[lane], wd.member[lane]);
+    __syncwarp();
   }
-  merge_candidates<NT>(a, s, sh);
+  __syncthreads();
 }
 
+// Scores n documents of a source; returns the number of candidates (the same in every thread).
 template <int G, int NT, class Src>
-__device__ __forceinline__ void eval(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, const Src &src,
-                                     int knn_stage) {
+__device__ __forceinline__ uint32_t score(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, const Src &src,
+                                          int knn_stage) {
   if constexpr (G == 1) {
     if (a.fp16) eval_wave_flat<NT, true>(a, s, sh, n, src, knn_stage);
     else eval_wave_flat<NT, false>(a, s, sh, n, src, knn_stage);
   } else {
     eval_wave<G, NT>(a, s, sh, n, src, knn_stage);
+  }
+  const uint32_t m = sh.ncand[s.turn];
+  s.turn ^= 1u;
+  return m;
+}
+
+// Takes a document of a wave back out of the seen set (its block turned out to be skipped).
+__device__ __forceinline__ void unsee(const SearchArgs &a, const Smem &s, uint32_t d) {
+  if (s.seen) {
+    atomicAnd(s.seen + (d >> 5), ~(1u << (d & 31)));
+    return;
+  }
+  uint32_t h = (d * 0x9E3779B1u) & (a.HS - 1u);
+  for (int p = 0; p < 16; p++) {
+    if (s.hash()[h] == d + 1u) {
+      s.hash()[h] = 0xFFFFFFFFu;  // no document's key, and not free: the probes behind it still find theirs
+      return;
+    }
+    h = (h + 1u) & (a.HS - 1u);
   }
 }
 
@@ -475,14 +702,17 @@ __device__ void bitonic_sort_u64(unsigned long long *keys, uint32_t P2) {
     }
 }
 
-// 5 CTAs of 256 threads per SM (48 registers).  A 40-register build for 6
-// CTAs per SM spilled little but measured 3-7 % slower at waves >= 4.
+// Lane groups: 5 CTAs of 256 threads per SM (48 registers).  Group 1: 4 CTAs (64
+// registers, two groups of units in flight without spills worth naming, 46 KB of
+// shared memory each); 5 CTAs at 48 registers, one group in flight and half the
+// filter took 68.7 ms where 4 take 65.6 (1M documents, 10k queries, cut 10).
 template <int G, int NW>
-__global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
+__global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
     k_search(const __grid_constant__ SearchArgs a) {
   constexpr int NT = NW * 32;
   __shared__ Shared sh;
-  Smem s{a, a.seen_bm ? a.seen_bm + (size_t)blockIdx.x * a.seen_words : nullptr};
+  Smem s{a, a.seen_bm ? a.seen_bm + (size_t)blockIdx.x * a.seen_words
+                      : a.seen_words ? reinterpret_cast<uint32_t *>(g_sm + a.off_hash) : nullptr, 0u};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   bool first = true;
 
@@ -503,6 +733,8 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
     const uint64_t qb = a.q_indptr[q], qe = a.q_indptr[q + 1];
     const uint32_t nnz = (uint32_t)(qe - qb);
     for (uint32_t i = tid; i < a.W; i += NT) s.qbits()[i] = 0u;
+    if (G == 1)
+      for (uint32_t i = tid; i < kFilter / 4; i += NT) reinterpret_cast<uint32_t *>(s.qfilt())[i] = 0u;
     if (s.seen) {  // seen_words is a multiple of 4 and the slot is 16-byte aligned
       uint4 *z = reinterpret_cast<uint4 *>(s.seen);
       for (uint32_t i = tid; i < a.seen_words / 4; i += NT) z[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -511,7 +743,7 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
     }
     if (tid < SEISMIC_STATS_N) sh.st[tid] = tid == SEISMIC_ST_T_START && a.stats ? globaltimer_ns() : 0ull;
     if (tid == 0) {
-      sh.count = 0; sh.ncand = 0; sh.nvalid = 0; sh.hash_full = 0; sh.bad = 0;
+      sh.count = 0; sh.ncand[0] = 0; sh.ncand[1] = 0; sh.nvalid = 0; sh.hash_full = 0; sh.hash_n = 0; sh.bad = 0;
       sh.cut = a.cut;
       sh.hf = a.hf;
       if (a.q_cut) {  // learned per-query parameters (already validated by their producer)
@@ -548,10 +780,10 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
         const uint32_t pos = s.qrank()[t >> 5] + __popc(w & ((1u << (t & 31)) - 1u));
         s.qval()[pos] = v;
         s.qterm()[pos] = (uint16_t)t;
+        if (G == 1) s.qfilt()[t & (kFilter - 1u)] = 1;
       }
     }
     __syncthreads();
-
     // ---------------------------------------------------------- H1: list terms
     if (a.alpha_q > 0.0f) {
       for (uint32_t i = tid; i < nzq; i += NT) {
@@ -610,9 +842,9 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
           sh.st[SEISMIC_ST_BLOCK_DOCS] += d1 - d0;
         }
         for (uint32_t c0 = d0; c0 < d1; c0 += a.CAND) {
-          const uint32_t n = min(a.CAND, d1 - c0);
-          const MemberSrc src{a.bdoc + c0, a.bdoc_row + c0};
-          eval<G, NT>(a, s, sh, n, src, 0);
+          const ListSrc src{nullptr, nullptr, 0u, c0, a.bdoc, a.bdoc_row};
+          const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, d1 - c0), src, 0);
+          if (m) merge_commit<NT>(s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
         }
         continue;
       }
@@ -623,15 +855,15 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
           words += summary_column(a.sbm, a.scptr, a.W, t, s.qterm()[i], s.clo() + i, s.chi() + i);
         if (a.stats && words) atomicAdd(&sh.st[SEISMIC_ST_DIR_LOOKUPS], (unsigned long long)words);
       }
-      for (uint32_t i = tid; i < NW * a.BMAX; i += NT) s.part()[i] = 0.0f;
+      for (uint32_t i = tid; i < a.NP * a.BMAX; i += NT) s.part()[i] = 0.0f;
       for (uint32_t b = tid; b <= nb; b += NT) s.bptr()[b] = __ldg(a.bdoc_ptr + g0 + b);  // block member ranges
       __syncthreads();
-      {
+      if ((uint32_t)warp < a.NP) {
         float *pw = s.part() + warp * a.BMAX;
         const float *bm = a.blk_m + g0;
         const float *bs = a.blk_size + g0;
         uint32_t ent = 0;
-        for (uint32_t i = warp; i < nzq; i += NW) {
+        for (uint32_t i = warp; i < nzq; i += a.NP) {
           const uint32_t lo = s.clo()[i], hi = s.chi()[i];
           const float qv = s.qval()[i];
           ent += hi - lo;
@@ -652,7 +884,7 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
       for (uint32_t b = tid; b < P2; b += NT) {
         if (b < nb) {
           float r = 0.0f;
-          for (int w = 0; w < NW; w++) r += s.part()[w * a.BMAX + b];
+          for (uint32_t w = 0; w < a.NP; w++) r += s.part()[w * a.BMAX + b];
           s.keys()[b] = ((unsigned long long)(~f2ord(r)) << 32) | b;
         } else {
           s.keys()[b] = ~0ull;
@@ -662,79 +894,118 @@ __global__ void __launch_bounds__(NW * 32, 1280 / (NW * 32))
       __syncthreads();
       // ---- H3: order blocks by (r desc, block asc)
       bitonic_sort_u64<NT>(s.keys(), P2);
-      // ---- H4/H5/H6: visit blocks in order, waves of a.wave blocks
+      // ---- H4/H5/H6: visit blocks in order.  A wave is the next W blocks that
+      // pass the test against theta (fewer past CAND documents; a larger block
+      // goes alone, in pieces).  Group 1 scores as many whole waves at once as
+      // fit CAND documents, as if theta stayed; when it rose so far that a later
+      // wave would have tested otherwise, the waves are merged one by one and
+      // what lies behind the first skip is undone.  So small waves cost a
+      // barrier and a round of memory latency per CAND documents, not per wave
+      // (300k documents, 2000 queries, wave 1: 21.1 ms; here 11.6).
       const uint32_t W = min(a.wave, kMaxWave);
+      const unsigned long long *keys = s.keys();
+      auto bscore = [&](uint32_t i) { return ord2f(~(uint32_t)(keys[i] >> 32)); };
+      auto limit = [&](float theta) { return a.hf_mode == 0 ? hf * theta : theta / hf; };
+      // the wave from block p on: its end, and its documents in nd
+      auto wave_end = [&](uint32_t p, uint32_t last, bool full, float thr, uint32_t &nd) {
+        uint32_t e = p;
+        nd = 0;
+        while (e < last && e - p < W) {
+          const uint32_t b = (uint32_t)(keys[e] & 0xFFFFFFFFu), bn = s.bptr()[b + 1] - s.bptr()[b];
+          if (e > p && ((full && bscore(e) < thr) || nd + bn > a.CAND)) break;
+          nd += bn;
+          e++;
+        }
+        return e;
+      };
       uint32_t bi = 0;
       while (bi < nb) {
         // skip test at the head of the wave (uniform: shared state after a barrier)
         const bool fullk = sh.count == a.k;
-        const float theta = fullk ? s.tk_s()[a.k - 1] : -INFINITY;
-        const float thr = a.hf_mode == 0 ? hf * theta : theta / hf;
-        if (fullk && ord2f(~(uint32_t)(s.keys()[bi] >> 32)) < thr) {
+        const float thr = fullk ? limit(s.tk_s()[a.k - 1]) : -INFINITY;
+        if (fullk && bscore(bi) < thr) {
           if (a.stats && tid == 0) sh.st[SEISMIC_ST_BLOCKS_SKIPPED] += nb - bi;
           break;
         }
-        // the wave: the next blocks that pass the test against theta now, up to
-        // W blocks and CAND documents (a larger block goes alone, in pieces)
-        uint32_t be = bi, ndocs = 0;
-        while (be < nb && be - bi < W) {
-          const uint32_t b = (uint32_t)(s.keys()[be] & 0xFFFFFFFFu);
-          if (be > bi && fullk && ord2f(~(uint32_t)(s.keys()[be] >> 32)) < thr) break;
-          const uint32_t nd = s.bptr()[b + 1] - s.bptr()[b];
-          if (be > bi && ndocs + nd > a.CAND) break;
+        uint32_t ndocs = 0;
+        const uint32_t first_end = wave_end(bi, nb, fullk, thr, ndocs);
+        uint32_t be = first_end;
+        while (G == 1 && be < nb && !(fullk && bscore(be) < thr)) {
+          uint32_t nd;
+          const uint32_t e = wave_end(be, nb, fullk, thr, nd);
+          if (ndocs + nd > a.CAND || e - bi > kMaxWave) break;
           ndocs += nd;
-          be++;
+          be = e;
         }
-        if (a.prefetch && tid < W && be + tid < nb) {  // member lists of the next wave's blocks
-          const uint32_t b = (uint32_t)(s.keys()[be + tid] & 0xFFFFFFFFu);
+        if (a.prefetch && tid < max(W, 8u) && be + tid < nb) {  // member lists of the next blocks
+          const uint32_t b = (uint32_t)(keys[be + tid] & 0xFFFFFFFFu);
           const uint32_t e0 = s.bptr()[b], e1 = s.bptr()[b + 1];
           prefetch_l2(a.bdoc + e0, 4 * (e1 - e0));
           prefetch_l2(a.bdoc_row + e0, 8 * (e1 - e0));
         }
-        if (a.stats && tid == 0) {
-          sh.st[SEISMIC_ST_BLOCKS_EVALUATED] += be - bi;
-          sh.st[SEISMIC_ST_BLOCK_DOCS] += ndocs;
-        }
-        if (be - bi == 1) {
-          const uint32_t b = (uint32_t)(s.keys()[bi] & 0xFFFFFFFFu);
-          const uint32_t d0 = s.bptr()[b], d1 = s.bptr()[b + 1];
-          for (uint32_t c0 = d0; c0 < d1; c0 += a.CAND) {
-            const MemberSrc src{a.bdoc + c0, a.bdoc_row + c0};
-            eval<G, NT>(a, s, sh, min(a.CAND, d1 - c0), src, 0);
+        uint32_t done = be, taken = ndocs;  // blocks up to here, and their documents, count
+        for (uint32_t c0 = 0; c0 < ndocs; c0 += a.CAND) {  // one round, unless a single block is larger
+          const ListSrc src{keys + bi, s.bptr(), be - bi, c0, a.bdoc, a.bdoc_row};
+          const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, ndocs - c0), src, 0);
+          if (m == 0) continue;
+          const uint32_t nc = merge_rank<NT>(a, s, sh, m, false, 0, 0);
+          if (be == first_end || nc < a.k || bscore(be - 1) >= limit(s.tmp_s()[a.k - 1])) {
+            merge_commit<NT>(s, sh, nc, true);
+            continue;
           }
-        } else {
-          const WaveBlocks src{s.keys() + bi, s.bptr(), be - bi, a.bdoc, a.bdoc_row};
-          eval<G, NT>(a, s, sh, ndocs, src, 0);
+          __syncthreads();  // everybody has read tmp
+          if (tid == 0) sh.nvalid = 0;
+          __syncthreads();
+          done = bi;
+          taken = 0;
+          while (done < be) {
+            const bool fk = sh.count == a.k;
+            const float th = fk ? limit(s.tk_s()[a.k - 1]) : -INFINITY;
+            if (fk && bscore(done) < th) break;
+            uint32_t nd;
+            const uint32_t e = wave_end(done, be, fk, th, nd);
+            merge_commit<NT>(s, sh, merge_rank<NT>(a, s, sh, m, true, taken, taken + nd), false);
+            taken += nd;
+            done = e;
+          }
+          for (uint32_t i = taken + tid; i < ndocs; i += NT)
+            if (s.fresh()[i]) {
+              uint32_t d;
+              unsigned long long row;
+              src.fetch(i, d, row);
+              unsee(a, s, d);
+              if (a.stats) {
+                atomicAdd(&sh.st[SEISMIC_ST_DOCS], ~0ull);
+                atomicAdd(&sh.st[SEISMIC_ST_DOC_NNZ], 0ull - (unsigned long long)a.fwd_nnz[d]);
+              }
+            }
+          if (tid == 0) sh.ncand[s.turn ^ 1u] = 0;
+          __syncthreads();
         }
-        bi = be;
+        if (a.stats && tid == 0) {
+          sh.st[SEISMIC_ST_BLOCKS_EVALUATED] += done - bi;
+          sh.st[SEISMIC_ST_BLOCK_DOCS] += taken;
+        }
+        bi = done;
       }
       __syncthreads();
     }
 
-    // graph refinement: the heap starts from the document and its neighbours
-    if (a.seed) {
-      const SeedSrc src{a.seed[q], a.knn, a.fwd_row, a.kappa, a.knn_bits};
-      eval<G, NT>(a, s, sh, 1 + a.kappa, src, 0);
-    }
-
+    // graph refinement starts the heap from the document and its neighbours; then
     // ---------------------------------------------------------- H7: kappa-NN expansion
-    if (a.use_knn && a.kappa > 0 && sh.count > 0) {
-      const uint32_t ns = sh.count;
-      for (uint32_t i = tid; i < ns; i += NT) s.clo()[i] = s.tk_id()[i];  // S, fixed before expanding
-      __syncthreads();
-      const uint32_t total = ns * a.kappa;
+    for (int stage = a.seed ? 0 : 1; stage < 2; stage++) {
+      uint32_t total = 1 + a.kappa;
+      if (stage == 1) {
+        const uint32_t ns = sh.count;
+        if (!(a.use_knn && a.kappa > 0 && ns > 0)) break;
+        for (uint32_t i = tid; i < ns; i += NT) s.clo()[i] = s.tk_id()[i];  // S, fixed before expanding
+        __syncthreads();
+        total = ns * a.kappa;
+      }
       for (uint32_t c0 = 0; c0 < total; c0 += a.CAND) {
-        const uint32_t n = min(a.CAND, total - c0);
-        const GraphSrc src{s.clo(), a.knn, a.fwd_row, a.kappa, a.knn_bits};
-        // positions c0 .. c0 + n of the neighbour list of S
-        struct Shifted {
-          GraphSrc g;
-          uint32_t c0;
-          __device__ uint32_t id(uint32_t i) const { return g.id(c0 + i); }
-          __device__ unsigned long long row(uint32_t i, uint32_t d) const { return g.row(c0 + i, d); }
-          __device__ void fetch(uint32_t i, uint32_t &d, unsigned long long &r) const { g.fetch(c0 + i, d, r); }
-        } sh_src{src, c0};
-        eval<G, NT>(a, s, sh, n, sh_src, 1);
+        const NeighbourSrc src{stage ? s.clo() : nullptr, a.knn, a.fwd_row, stage ? 0u : a.seed[q], a.kappa, a.knn_bits, c0};
+        const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, total - c0), src, stage);
+        if (m) merge_commit<NT>(s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
       }
     }
 
@@ -785,7 +1056,8 @@ size_t search_layout(SearchArgs &a, uint32_t nw) {
   a.off_qterm = take(a.QN * 2);
   a.off_cut = take(a.QN * 2);
   a.off_aq = take(a.alpha_q > 0.0f ? a.QN * 4 : 4);
-  a.off_part = take(a.exhaustive ? 4 : nw * a.BMAX * 4);
+  if (!a.NP) a.NP = nw;
+  a.off_part = take(a.exhaustive ? 4 : a.NP * a.BMAX * 4);
   a.off_keys = take(a.exhaustive ? 8 : a.BPOW2 * 8);
   const uint32_t nclo = std::max(a.QN, a.k);  // clo also holds S during the expansion
   a.off_clo = take(nclo * 4);
@@ -798,27 +1070,35 @@ size_t search_layout(SearchArgs &a, uint32_t nw) {
   a.off_cand_s = take(a.CAND * 4);
   a.off_cand_id = take(a.CAND * 4);
   a.off_cand_ok = take(a.CAND);
+  a.off_cand_i = take(a.flat ? a.CAND * 2 : 0);
+  a.off_fresh = take(a.flat ? a.CAND : 0);
   a.off_bptr = take(a.exhaustive ? 4 : (a.BMAX + 1) * 4);
-  a.CAPC = 0;
   if (a.flat) {
-    // chunk partials reuse the block-score partials; at least 2048 chunks,
-    // more than any row holds (kMaxRowNnzBuild / kChunk)
-    a.CAPC = std::max<uint32_t>(2048u, (a.exhaustive ? 0u : nw * a.BMAX));
-    if (a.exhaustive || nw * a.BMAX < a.CAPC) {
-      a.off_part = take(a.CAPC * 4);  // the earlier part region is too small: a fresh one
-    }
-    a.off_fdoc = take(a.CAND * 4);
-    a.off_fc0 = take(a.CAND * 4);
-    a.off_fpre = take((a.CAND + 1) * 4);
-    a.off_cmap = take(a.CAPC);
+    // the warps' candidate queues: in the block-score partials' space (dead
+    // while documents are scored) where they fit
+    const uint32_t queues = nw * kWarpQueueBytes;
+    a.off_wqueue = a.off_keys - a.off_part >= queues ? a.off_part : take(queues);
+    a.off_qfilt = take(kFilter);
+    a.off_wdocs = take(nw * kWarpDocsBytes);
   }
   return o;
+}
+
+// A query alone on its SM is bound by latency: the more warps share a wave's
+// documents, the fewer loads follow one another.  One CTA of 32 warps per SM up
+// to as many queries as SMs, 16 warps up to twice that, else 8 (one query, 1M documents, cut 10: 3.0 ms with 8 warps, 2.4 with
+// 32; 1000 queries, 100k documents: 2.6 ms with 8, 3.2 with 16).
+// The block scores are added up as by 8 warps in each (SearchArgs::NP), so the
+// results do not depend on the choice.
+uint32_t search_warps(uint32_t group, uint32_t asked, uint32_t nq, uint32_t sms) {
+  if (asked) return asked;
+  return group != 1 || nq > 2 * sms ? 8u : nq > sms ? 16u : 32u;
 }
 
 int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, uint32_t grid, cudaStream_t st) {
 #define SZ_CASE(G_, NW_) \
   if (group == G_ && nw == NW_) return launch_t<G_, NW_>(a, smem, grid, st);
-  SZ_CASE(1, 4) SZ_CASE(1, 8) SZ_CASE(1, 16)
+  SZ_CASE(1, 4) SZ_CASE(1, 8) SZ_CASE(1, 16) SZ_CASE(1, 32)
   SZ_CASE(8, 4) SZ_CASE(8, 8) SZ_CASE(8, 16)
   SZ_CASE(16, 4) SZ_CASE(16, 8) SZ_CASE(16, 16)
   SZ_CASE(32, 4) SZ_CASE(32, 8) SZ_CASE(32, 16)
@@ -829,7 +1109,7 @@ int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem,
 int search_occupancy(uint32_t group, uint32_t nw, size_t smem, int *blocks) {
 #define SZ_CASE(G_, NW_) \
   if (group == G_ && nw == NW_) return occupancy_t<G_, NW_>(smem, blocks);
-  SZ_CASE(1, 4) SZ_CASE(1, 8) SZ_CASE(1, 16)
+  SZ_CASE(1, 4) SZ_CASE(1, 8) SZ_CASE(1, 16) SZ_CASE(1, 32)
   SZ_CASE(8, 4) SZ_CASE(8, 8) SZ_CASE(8, 16)
   SZ_CASE(16, 4) SZ_CASE(16, 8) SZ_CASE(16, 16)
   SZ_CASE(32, 4) SZ_CASE(32, 8) SZ_CASE(32, 16)

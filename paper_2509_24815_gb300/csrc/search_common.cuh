@@ -38,22 +38,27 @@ __device__ __forceinline__ float qlookup(const uint32_t *__restrict__ qbits, con
   return qval[qrank[t >> 5] + __popc(w & (bit - 1u))];
 }
 
-// 16-byte read-only load that does not allocate in L1 (rows are read once per
-// query; reuse across queries is in L2)
+// Read-only loads that do not allocate in L1 (rows are read once per query;
+// reuse across queries is in L2) and fetch 64 bytes, not a whole 128-byte line,
+// from DRAM on a miss: a scattered 32-byte read moved 124 bytes from DRAM
+// without the L2::64B qualifier and 63 with it (3 GB buffer).  ldg_na reads 16
+// bytes, ldg_na_v8 32 bytes (one sector; p is 32-byte aligned), ldg_na_f32 one float.
 __device__ __forceinline__ uint4 ldg_na(const void *p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;
 }
-
-// 32-byte read-only load (one DRAM sector) that does not allocate in L1; p is
-// 32-byte aligned
 __device__ __forceinline__ void ldg_na_v8(const void *p, uint4 &lo, uint4 &hi) {
-  asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
                : "l"(p));
+}
+__device__ __forceinline__ float ldg_na_f32(unsigned long long p) {
+  float r;
+  asm volatile("ld.global.nc.L1::no_allocate.L2::64B.f32 %0, [%1];" : "=f"(r) : "l"(p));
+  return r;
 }
 
 // TMA bulk prefetch of [p, p + bytes) into L2 (no registers, no completion):
@@ -193,23 +198,6 @@ struct GraphSrc {  // the kappa-NN neighbours of the ids in S
   __device__ __forceinline__ void fetch(uint32_t x, uint32_t &d, unsigned long long &r) const {
     d = id(x);
     r = row(x, d);
-  }
-};
-
-struct SeedSrc {  // a document, then its kappa-NN neighbours
-  uint32_t doc;
-  const uint32_t *knn;
-  const unsigned long long *frow;
-  uint32_t kappa, bits;
-  __device__ __forceinline__ uint32_t id(uint32_t i) const {
-    return i == 0 ? doc : knn_entry(knn, bits, (uint64_t)doc * kappa + (i - 1));
-  }
-  __device__ __forceinline__ unsigned long long row(uint32_t, uint32_t d) const {
-    return d == SEISMIC_NONE_ID ? 0ull : __ldg(frow + d);
-  }
-  __device__ __forceinline__ void fetch(uint32_t i, uint32_t &d, unsigned long long &r) const {
-    d = id(i);
-    r = row(i, d);
   }
 };
 

@@ -220,6 +220,8 @@ int seismic_server_create(seismic_index *ix, const seismic_search_params *search
     std::unique_ptr<seismic_server> srv(new seismic_server());
     srv->ix = ix;
     srv->sp = *search;
+    // batches share the GPU: the shape that suits a full one, whatever a batch's size
+    if (!srv->sp.cta_warps && search->shape != 2) srv->sp.cta_warps = 8;
     if (params) srv->pp = *params;
     if (!srv->pp.max_batch) srv->pp.max_batch = 256;
     if (!srv->pp.streams) srv->pp.streams = 4;
@@ -236,7 +238,7 @@ int seismic_server_create(seismic_index *ix, const seismic_search_params *search
       a.BPOW2 = 1;
       while (a.BPOW2 < a.BMAX) a.BPOW2 <<= 1;
       a.HS = 16;
-      a.CAND = 256;
+      a.CAND = kCand;
       a.k = std::max<uint32_t>(search->k, 100);
       a.alpha_q = search->alpha_q;
       const uint32_t nw = search->cta_warps ? search->cta_warps : 8, g = search->group ? search->group : 1;

@@ -77,3 +77,56 @@ def test_mlp_gradient_row_edges(sz, n, offset):
     assert np.linalg.norm(got - ref) <= 1e-2 * np.linalg.norm(ref)
     assert abs(loss.item() - (e * e).sum() / n) <= 1e-3 * loss.item()
     np.testing.assert_array_equal(buf[0].cpu().numpy(), w)  # learning rate 0
+
+
+@pytest.fixture(scope="module", params=[False, True], ids=["fp32", "fp16"])
+def dense_hits(sz, request):
+    """Whole-valued rows and queries over few terms, so that a row's terms are mostly hits (the candidate queues
+    fill), with rows of 1..40 entries, of 300..500, beyond a queue's 2048 positions, and copies of queries."""
+    dim = 4000
+    short, mid = _int_rows(2500, 300, 1, 40, -1, 4, 11), _int_rows(300, 600, 300, 500, -1, 4, 12)
+    long, queries = _int_rows(7, dim, 2049, 2600, 1, 4, 13), _int_rows(330, 520, 1, 400, 1, 3, 14)
+    parts = [short, mid, long, queries.slice(0, 60)]
+    indptr = np.concatenate([[0]] + [np.diff(p.indptr.astype(np.int64)) for p in parts]).cumsum().astype(np.uint64)
+    docs = synth.CSR(indptr, np.concatenate([p.terms for p in parts]), np.concatenate([p.vals for p in parts]), dim)
+    queries = synth.CSR(queries.indptr, queries.terms, queries.vals, dim)
+    ix = sz.seismic_build(docs, lambda_=400, beta=60, alpha=0.6, quantize_u8=False, seed=2, values_fp16=request.param)
+    yield docs, queries, ix
+    ix.close()
+
+
+# Lane groups score one row at a time and one wave at a time; sums of whole values are exact in any order, so the
+# documents, the scores and the work counted have to be the same.
+@pytest.mark.parametrize("kw", [dict(wave=1), dict(wave=1, heap_factor=1.3), dict(wave=3, heap_factor=1.0),
+                                dict(wave=2, hf_mode=1, heap_factor=0.8), dict(wave=64), dict(exhaustive=True)],
+                         ids=lambda d: ",".join(f"{k}={v}" for k, v in d.items()))
+@pytest.mark.parametrize("launch", [dict(persistent=True), dict(persistent=True, cta_warps=4), dict(persistent=False),
+                                    dict(persistent=False, hash_slots=16)],
+                         ids=["persistent", "4 warps", "plain", "tiny hash"])
+@pytest.mark.parametrize("nq,k", [(1, 3), (200, 10), (330, 60)])
+def test_group_1_equals_lane_groups(sz, dense_hits, kw, launch, nq, k):
+    _, queries, ix = dense_hits
+    q = queries.slice(0, nq)
+    kw = dict(dict(cut=9, heap_factor=0.9), k=k, **kw) if "heap_factor" not in kw else dict(cut=9, k=k, **kw)
+    gi, gs, gst = sz.seismic_search(ix, q, group=1, stats=True, **launch, **kw)
+    ri, rs, rst = sz.seismic_search(ix, q, group=32, cta_warps=8, persistent=True, stats=True, **kw)
+    np.testing.assert_array_equal(gs, rs)
+    np.testing.assert_array_equal(gi, ri)
+    for name in ("lists", "blocks_scored", "blocks_evaluated", "blocks_skipped", "block_docs", "summary_entries"):
+        np.testing.assert_array_equal(gst[:, sz.STATS.index(name)], rst[:, sz.STATS.index(name)], err_msg=name)
+    if "hash_slots" not in launch:  # a set that forgets scores some documents again
+        for name in ("docs", "doc_nnz"):
+            np.testing.assert_array_equal(gst[:, sz.STATS.index(name)], rst[:, sz.STATS.index(name)], err_msg=name)
+
+
+def test_group_1_graph_stages_equal_lane_groups(sz, dense_hits):
+    docs, queries, ix = dense_hits
+    rng = np.random.default_rng(5)
+    sz.seismic_set_knn(ix, rng.integers(0, docs.n_rows, (docs.n_rows, 7)))
+    for launch in (dict(persistent=True), dict(persistent=False, hash_slots=16)):
+        for nq in (3, 330):
+            got = sz.seismic_search(ix, queries.slice(0, nq), k=50, cut=2, heap_factor=1.0, use_knn=True, **launch)
+            ref = sz.seismic_search(ix, queries.slice(0, nq), k=50, cut=2, heap_factor=1.0, use_knn=True, group=16,
+                                    persistent=True)
+            np.testing.assert_array_equal(got[1], ref[1])
+            np.testing.assert_array_equal(got[0], ref[0])
