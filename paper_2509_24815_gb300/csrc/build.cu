@@ -129,7 +129,7 @@ uint64_t splitmix64_next(uint64_t &state) {
 // sequential merge of the two sorted rows.  Argmax ties keep the lower
 // centroid index.
 constexpr int kAsgThreads = 128;
-constexpr int kAsgCC = 48;        // centroids per chunk (cluster index fits in u8); 2 CTAs per SM
+constexpr int kAsgCC = 50;        // centroids per chunk (cluster index fits in u8); as many as leave 2 CTAs per SM
 constexpr int kAsgMaxEnt = 8192;  // nonzeros per chunk (= kMaxRowNnzBuild bound below)
 static_assert(kMaxRowNnzBuild <= kAsgMaxEnt, "a centroid row must fit one chunk");
 static_assert((size_t)kAsgCC * kAsgThreads * 8 >= (size_t)(kAsgMaxEnt + 1) * 4, "the cursors share the accumulators");
@@ -273,14 +273,29 @@ __global__ void __launch_bounds__(kAsgThreads) k_assign(
       for (uint32_t i = tid; i < n; i += kAsgThreads) {
         const uint32_t j = list_doc[lp0 + i];
         for (uint32_t cc = 0; cc < ncc; cc++) a[cc * kAsgThreads] = 0.0;
-        // the member's terms in ascending order, 8 per 16-byte load from its
-        // forward-index record; a value is read only where the chunk holds the term
+        // the member's terms in ascending order, 8 at a time with their values, the next 8 read while these
+        // are scored (read behind their terms, with 48 centroids per chunk: 0.43 s where this takes 0.39, 100k documents, 100 blocks)
         const unsigned long long row = fwd_row[j];
         const uint8_t *rec = fwd + (size_t)(uint32_t)row * kUnitBytes;
         const uint32_t nch = (uint32_t)(row >> 32), nnz = (uint32_t)(indptr[j + 1] - indptr[j]);
+        auto fetch = [&](uint32_t o, uint4 &t, uint4 &x, uint4 &y) {
+          if (o >= nch) return;
+          if (fp16) {
+            t = *reinterpret_cast<const uint4 *>(rec + (size_t)o * kUnitBytes);
+            x = *reinterpret_cast<const uint4 *>(rec + (size_t)o * kUnitBytes + 16);
+          } else {
+            t = *reinterpret_cast<const uint4 *>(rec + (size_t)o * 16u);
+            const uint4 *v = reinterpret_cast<const uint4 *>(rec + (size_t)kUnitBytes * ((nch + 1) / 2 + o));
+            x = v[0];
+            y = v[1];
+          }
+        };
+        uint4 tn = make_uint4(0u, 0u, 0u, 0u), xn = tn, yn = tn;
+        fetch(0, tn, xn, yn);
         for (uint32_t o = 0; o < nch; o++) {
-          const uint4 tq = *reinterpret_cast<const uint4 *>(rec + (size_t)o * (fp16 ? kUnitBytes : 16u));
-          const uint32_t tw[4] = {tq.x, tq.y, tq.z, tq.w};
+          const uint32_t tw[4] = {tn.x, tn.y, tn.z, tn.w};
+          const uint32_t vw[8] = {xn.x, xn.y, xn.z, xn.w, yn.x, yn.y, yn.z, yn.w};
+          fetch(o + 1, tn, xn, yn);
 #pragma unroll
           for (uint32_t e8 = 0; e8 < kChunk; e8++) {
             if (o * kChunk + e8 >= nnz) break;  // the padding after the row's last entry
@@ -289,12 +304,9 @@ __global__ void __launch_bounds__(kAsgThreads) k_assign(
             const uint32_t bit = 1u << (s & 31);
             if (!(w & bit)) continue;
             const uint32_t idx = crank[s >> 5] + __popc(w & (bit - 1u));
-            double u;
-            if (fp16) {
-              u = (double)__half2float(*reinterpret_cast<const __half *>(rec + (size_t)o * kUnitBytes + 16 + 2 * e8));
-            } else {
-              u = (double)*reinterpret_cast<const float *>(rec + (size_t)kUnitBytes * ((nch + 1) / 2 + o) + 4 * e8);
-            }
+            const double u =
+                fp16 ? (double)__half2float(__ushort_as_half((unsigned short)((e8 & 1) ? (vw[e8 >> 1] >> 16) : (vw[e8 >> 1] & 0xFFFFu))))
+                     : (double)__uint_as_float(vw[e8]);
             for (uint32_t e = coff[idx]; e < coff[idx + 1]; e++)
               a[(uint32_t)ent_c[e] * kAsgThreads] = __dadd_rn(a[(uint32_t)ent_c[e] * kAsgThreads],
                                                                 __dmul_rn(u, (double)ent_w[e]));

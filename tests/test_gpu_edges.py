@@ -130,3 +130,51 @@ def test_group_1_graph_stages_equal_lane_groups(sz, dense_hits):
                                     persistent=True)
             np.testing.assert_array_equal(got[1], ref[1])
             np.testing.assert_array_equal(got[0], ref[0])
+
+
+# Masses spread over more than 53 bits are added one after the other, others as integers: both give the prefix of
+# sequential fp64 sums.  Codes are quantised in fp64 from the kept values.
+@pytest.mark.parametrize("spread", [0, 12, 40])
+@pytest.mark.parametrize("alpha", [0.05, 0.4, 1.0])
+def test_summary_masses_and_codes(sz, spread, alpha):
+    rng = np.random.default_rng(spread)
+    docs = _int_rows(700, 3000, 1, 300, 1, 3, 21)
+    vals = (rng.random(docs.nnz) + 0.5) * np.exp2(rng.integers(-spread, 1, docs.nnz)) * rng.choice([1, 1, 1, -1], docs.nnz)
+    docs = synth.CSR(docs.indptr, docs.terms, vals.astype(np.float32), docs.dim)
+    ix = sz.seismic_build(docs, lambda_=60, beta=7, alpha=alpha, quantize_u8=True, seed=1, keep_block_summaries=True)
+    x = {n: sz.seismic_export(ix, n) for n in ("bdoc_ptr", "bdoc", "sum_ptr", "sum_term", "sum_val", "sum_code")}
+    ix.close()
+    dense = docs.to_dense()
+    blocks = rng.choice(len(x["bdoc_ptr"]) - 1, 400, replace=False)
+    for g in blocks:
+        phi = dense[x["bdoc"][x["bdoc_ptr"][g]:x["bdoc_ptr"][g + 1]]].max(axis=0)
+        order = np.lexsort((np.arange(docs.dim), -np.abs(phi)))
+        order = order[phi[order] != 0]
+        mass = np.cumsum(np.abs(phi[order]))
+        keep = order[:int(np.argmax(mass >= alpha * mass[-1])) + 1] if len(order) else order
+        a, b = int(x["sum_ptr"][g]), int(x["sum_ptr"][g + 1])
+        keep = np.sort(keep)
+        np.testing.assert_array_equal(x["sum_term"][a:b], keep)
+        np.testing.assert_array_equal(x["sum_val"][a:b], phi[keep].astype(np.float32))
+        if len(keep):
+            m, size = phi[keep].min(), float(np.float32((phi[keep].max() - phi[keep].min()) / 256.0))
+            code = np.clip(np.floor((phi[keep] - m) / size), 0, 255) if size > 0 else np.zeros(len(keep))
+            np.testing.assert_array_equal(x["sum_code"][a:b], code.astype(np.uint8))
+
+
+# A shared-memory budget that holds for the query alone: long queries leave group 1 for lane groups, past 200 KB
+# they are refused, whatever the seen set.
+def test_long_queries_and_the_shared_memory_limit(sz):
+    dim = 40000
+    docs = _int_rows(500, dim, 1000, 3000, 1, 3, 31)
+    q = _int_rows(3, dim, 6000, 9000, 1, 2, 32)
+    ix = sz.seismic_build(docs, lambda_=50, beta=5, alpha=0.5, quantize_u8=False, seed=1)
+    for kw in (dict(), dict(persistent=True), dict(cta_warps=16), dict(hash_slots=64)):
+        got = sz.seismic_search(ix, q, k=5, cut=40, heap_factor=1.0, **kw)
+        ref = sz.seismic_search(ix, q, k=5, cut=40, heap_factor=1.0, group=8, persistent=True, cta_warps=kw.get("cta_warps", 8))
+        np.testing.assert_array_equal(got[1], ref[1])
+        np.testing.assert_array_equal(got[0], ref[0])
+    with pytest.raises(sz.SeismicError) as e:
+        sz.seismic_search(ix, _int_rows(2, dim, 14000, 15000, 1, 2, 33), k=5, cut=40)
+    assert e.value.code == sz.EBUDGET
+    ix.close()
