@@ -292,9 +292,7 @@ int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const
     a.QN = std::max<uint32_t>(a.QN, 32);
   }
   // defaults: one CTA per query with chunk-flattened scoring (the measured fastest)
-  const uint32_t group = p->group ? p->group : (p->shape == 2 ? 8 : 1);
-  uint32_t nw = search_warps(group, p->cta_warps, nq, (uint32_t)sm_count(ix->device));
-  a.NP = p->cta_warps ? p->cta_warps : 8;
+  uint32_t group = p->group ? p->group : (p->shape == 2 ? 8 : 1);
   a.sum_absmax = ix->sum_absmax;
   a.prefetch = p->no_prefetch ? 0u : 256u;
   const bool warp_shape0 = p->shape == 2;
@@ -330,28 +328,23 @@ int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const
     a.persistent = 1;
     if ((rc = launch_search_warp(a, group, smem, grid, wpb, st))) return rc;
   } else {
-  a.flat = group == 1 ? 1u : 0u;
   // a small collection's seen set fits shared memory as a bitmap, exact and one atomic per
   // document (100k documents, 12.5 KB: 1000 queries 2.0 ms; the hash set 2.5)
-  if (a.flat && !a.persistent && !p->hash_slots && ix->n_docs <= kSeenDocs) {
-    a.seen_words = (uint32_t)(((ix->n_docs + 31) / 32 + 3) & ~3ull);
-    a.HS = a.seen_words;
-  }
-  size_t smem = search_layout(a, nw);
-  if (smem > 200 * 1024 && !p->cta_warps) smem = search_layout(a, nw = 8);
-  if (smem > 200 * 1024)
-    return fail(SEISMIC_EBUDGET, "search: shared memory per query (" + std::to_string(smem) +
+  const uint32_t words = (uint32_t)(((ix->n_docs + 31) / 32 + 3) & ~3ull);
+  uint32_t nw = 8;
+  const size_t smem = search_fit(a, group, p->cta_warps, (uint32_t)sm_count(ix->device),
+                                 !a.persistent && !p->hash_slots && ix->n_docs <= kSeenDocs ? words : 0u, nw);
+  if (smem == 0)
+    return fail(SEISMIC_EBUDGET, "search: shared memory per query (" + std::to_string(a.budget) +
                                      " B) exceeds 200 KB; lower hash_slots or the query size");
   uint32_t grid = nq;
   if (a.persistent) {
     // persistent CTAs keep a seen bitmap of the collection each, in global
     // memory (cleared per query), so deduplication never overflows
-    a.HS = 16;
-    smem = search_layout(a, nw);
     int blocks = 1;
     if ((rc = search_occupancy(group, nw, smem, &blocks))) return rc;
     grid = (uint32_t)std::min<uint64_t>(nq, (uint64_t)std::max(1, blocks) * sm_count(ix->device));
-    a.seen_words = (uint32_t)(((ix->n_docs + 31) / 32 + 3) & ~3ull);
+    a.seen_words = words;
     if ((rc = w->seen.ensure((size_t)grid * a.seen_words * 4))) return rc;
     a.seen_bm = w->seen.as<uint32_t>();
   }
@@ -457,6 +450,47 @@ int set_knn_impl(seismic_index *ix, const uint32_t *nbrs, uint64_t n, uint32_t k
   return SEISMIC_OK;
 }
 
+// One device allocation for a graph pass's buffers (five or six of them,
+// allocated and freed one by one, took a millisecond per call).
+struct GraphBufs {
+  DevBuf all;
+  uint64_t *ip = nullptr;
+  uint16_t *tt = nullptr;
+  float *vv = nullptr, *sc = nullptr;
+  uint32_t *ids = nullptr, *seeds = nullptr;
+  // rows: documents of a batch at most; entries: padded row entries of a batch at most
+  int alloc(uint64_t rows, uint64_t entries, uint32_t kk) {
+    size_t o = 0;
+    auto take = [&](size_t n) {
+      const size_t at = o;
+      o += (n + 255) & ~(size_t)255;
+      return at;
+    };
+    const size_t a = take((rows + 1) * 8), b = take(entries * 2 + 16), c = take(entries * 4 + 16), d = take(rows * kk * 4),
+                 e = take(rows * kk * 4), f = take(rows * 4);
+    if (int rc = all.alloc(o)) return rc;
+    uint8_t *p = all.as<uint8_t>();
+    ip = reinterpret_cast<uint64_t *>(p + a);
+    tt = reinterpret_cast<uint16_t *>(p + b);
+    vv = reinterpret_cast<float *>(p + c);
+    ids = reinterpret_cast<uint32_t *>(p + d);
+    sc = reinterpret_cast<float *>(p + e);
+    seeds = reinterpret_cast<uint32_t *>(p + f);
+    return SEISMIC_OK;
+  }
+};
+
+// The padded entries of the largest batch of rows.
+uint64_t largest_batch(const std::vector<uint64_t> &frow, uint64_t batch) {
+  uint64_t most = 0;
+  for (uint64_t r0 = 0; r0 < frow.size(); r0 += batch) {
+    uint64_t e = 0;
+    for (uint64_t i = r0; i < std::min<uint64_t>(frow.size(), r0 + batch); i++) e += 8u * (uint32_t)(frow[i] >> 32);
+    most = std::max(most, e);
+  }
+  return most;
+}
+
 // kappa-NN graph of the collection itself: exact (params NULL, needs the
 // unpruned lists) or with Seismic search as the paper builds it.  Each
 // document is a query; the top kappa+1 minus the document itself remain.
@@ -469,13 +503,13 @@ int build_knn_impl(seismic_index *ix, uint32_t kappa, const seismic_search_param
   const uint32_t kk = kappa + 1;
   const uint64_t batch = 1u << 16;
   std::vector<uint32_t> graph(N * kappa, SEISMIC_NONE_ID);
-  DevBuf ip, tt, vv, ids, sc;
   std::vector<uint64_t> frow(N), hip(batch + 1);
   SZ_CUDA(cudaMemcpy(frow.data(), ix->fwd_row.p, N * 8, cudaMemcpyDeviceToHost));
+  const uint64_t rows = std::min<uint64_t>(batch, N);
+  GraphBufs b;
   int rc;
-  if ((rc = ids.alloc(batch * kk * 4)) || (rc = sc.alloc(batch * kk * 4)) || (rc = ip.alloc((batch + 1) * 8)))
-    return rc;
-  std::vector<uint32_t> hid(batch * kk);
+  if ((rc = b.alloc(rows, largest_batch(frow, batch), kk))) return rc;
+  std::vector<uint32_t> hid(rows * kk);
   seismic_search_params sp{};
   if (p) {
     sp = *p;
@@ -493,22 +527,20 @@ int build_knn_impl(seismic_index *ix, uint32_t kappa, const seismic_search_param
       hip[i + 1] = hip[i] + e;
       mx = std::max(mx, e);
     }
-    const uint64_t ent = hip[n];
-    if ((rc = tt.ensure(ent * 2 + 16)) || (rc = vv.ensure(ent * 4 + 16))) return rc;
-    SZ_CUDA(cudaMemcpy(ip.p, hip.data(), (n + 1) * 8, cudaMemcpyHostToDevice));
+    SZ_CUDA(cudaMemcpy(b.ip, hip.data(), (n + 1) * 8, cudaMemcpyHostToDevice));
     k_fwd_to_csr<<<(unsigned)std::min<uint64_t>(n, 65535), 64>>>(ix->fwd_row.as<unsigned long long>(),
                                                                  ix->fwd_data.as<uint8_t>(), ix->bp.values_fp16, r0, n,
-                                                                 ip.as<uint64_t>(), tt.as<uint16_t>(), vv.as<float>());
+                                                                 b.ip, b.tt, b.vv);
     SZ_CUDA(cudaGetLastError());
-    seismic_csr qc{ip.as<uint64_t>(), tt.as<uint16_t>(), vv.as<float>(), n, ix->dim, 1};
+    seismic_csr qc{b.ip, b.tt, b.vv, n, ix->dim, 1};
     if (p) {
       sp.max_query_nnz = mx;
-      rc = search_impl(ix, &qc, &sp, ids.as<uint32_t>(), sc.as<float>(), 1, nullptr, nullptr);
+      rc = search_impl(ix, &qc, &sp, b.ids, b.sc, 1, nullptr, nullptr);
     } else {
-      rc = exact_impl(ix, &qc, kk, ids.as<uint32_t>(), sc.as<float>(), 1, nullptr);
+      rc = exact_impl(ix, &qc, kk, b.ids, b.sc, 1, nullptr);
     }
     if (rc) return rc;
-    SZ_CUDA(cudaMemcpy(hid.data(), ids.p, n * kk * 4, cudaMemcpyDeviceToHost));
+    SZ_CUDA(cudaMemcpy(hid.data(), b.ids, n * kk * 4, cudaMemcpyDeviceToHost));
     for (uint64_t i = 0; i < n; i++) {
       uint32_t self = (uint32_t)(r0 + i), o = 0;
       for (uint32_t j = 0; j < kk && o < kappa; j++) {
@@ -536,12 +568,11 @@ int refine_knn_impl(seismic_index *ix, uint32_t rounds, const seismic_search_par
   const uint32_t kappa = ix->kappa, kk = kappa + 1;
   std::vector<uint64_t> frow(N), hip(batch + 1);
   SZ_CUDA(cudaMemcpy(frow.data(), ix->fwd_row.p, N * 8, cudaMemcpyDeviceToHost));
-  DevBuf ip, tt, vv, ids, sc, seeds;
+  const uint64_t rows = std::min<uint64_t>(batch, N);
+  GraphBufs b;
   int rc;
-  if ((rc = ids.alloc(batch * kk * 4)) || (rc = sc.alloc(batch * kk * 4)) || (rc = ip.alloc((batch + 1) * 8)) ||
-      (rc = seeds.alloc(batch * 4)))
-    return rc;
-  std::vector<uint32_t> hid(batch * kk), hseed(batch);
+  if ((rc = b.alloc(rows, largest_batch(frow, batch), kk))) return rc;
+  std::vector<uint32_t> hid(rows * kk), hseed(rows);
   seismic_search_params sp{};
   if (p) sp = *p;
   sp.k = kk;
@@ -565,20 +596,16 @@ int refine_knn_impl(seismic_index *ix, uint32_t rounds, const seismic_search_par
         mx = std::max(mx, e);
         hseed[i] = (uint32_t)(r0 + i);
       }
-      if ((rc = tt.ensure(hip[n] * 2 + 16)) || (rc = vv.ensure(hip[n] * 4 + 16))) return rc;
-      SZ_CUDA(cudaMemcpy(ip.p, hip.data(), (n + 1) * 8, cudaMemcpyHostToDevice));
-      SZ_CUDA(cudaMemcpy(seeds.p, hseed.data(), n * 4, cudaMemcpyHostToDevice));
+      SZ_CUDA(cudaMemcpy(b.ip, hip.data(), (n + 1) * 8, cudaMemcpyHostToDevice));
+      SZ_CUDA(cudaMemcpy(b.seeds, hseed.data(), n * 4, cudaMemcpyHostToDevice));
       k_fwd_to_csr<<<(unsigned)std::min<uint64_t>(n, 65535), 64>>>(ix->fwd_row.as<unsigned long long>(),
                                                                    ix->fwd_data.as<uint8_t>(), ix->bp.values_fp16, r0,
-                                                                   n, ip.as<uint64_t>(), tt.as<uint16_t>(),
-                                                                   vv.as<float>());
+                                                                   n, b.ip, b.tt, b.vv);
       SZ_CUDA(cudaGetLastError());
-      seismic_csr qc{ip.as<uint64_t>(), tt.as<uint16_t>(), vv.as<float>(), n, ix->dim, 1};
+      seismic_csr qc{b.ip, b.tt, b.vv, n, ix->dim, 1};
       sp.max_query_nnz = mx;
-      if ((rc = search_ws(ix, &ix->ws, &qc, &sp, ids.as<uint32_t>(), sc.as<float>(), 1, nullptr, nullptr,
-                          seeds.as<uint32_t>())))
-        return rc;
-      SZ_CUDA(cudaMemcpy(hid.data(), ids.p, n * kk * 4, cudaMemcpyDeviceToHost));
+      if ((rc = search_ws(ix, &ix->ws, &qc, &sp, b.ids, b.sc, 1, nullptr, nullptr, b.seeds))) return rc;
+      SZ_CUDA(cudaMemcpy(hid.data(), b.ids, n * kk * 4, cudaMemcpyDeviceToHost));
       for (uint64_t i = 0; i < n; i++) {
         const uint32_t self = (uint32_t)(r0 + i);
         uint32_t o = 0;

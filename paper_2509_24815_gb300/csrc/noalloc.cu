@@ -58,8 +58,7 @@ extern "C" int seismic_search_noalloc(seismic_index *ix, const seismic_csr *quer
   if (p->use_knn && ix->kappa == 0) return fail(SEISMIC_EINVAL, "use_knn: the index has no kappa-NN graph");
   if (p->shape == 2) return fail(SEISMIC_EINVAL, "noalloc search: only the CTA-per-query shape (0 or 1)");
   if (p->shape > 2) return fail(SEISMIC_EINVAL, "shape must be 0 (auto), 1 (CTA per query) or 2 (warp per query)");
-  const uint32_t group = p->group ? p->group : 1;
-  uint32_t nw = p->cta_warps ? p->cta_warps : 8;
+  uint32_t group = p->group ? p->group : 1, nw = p->cta_warps ? p->cta_warps : 8;
   if (!(group == 1 || group == 8 || group == 16 || group == 32) || !(nw == 4 || nw == 8 || nw == 16))
     return fail(SEISMIC_EINVAL, "noalloc search: group must be 1/8/16/32 and cta_warps 4/8/16");
   if (queries->n_rows == 0) return SEISMIC_OK;
@@ -128,14 +127,10 @@ extern "C" int seismic_search_noalloc(seismic_index *ix, const seismic_csr *quer
   a.sum_absmax = ix->sum_absmax;
   a.prefetch = p->no_prefetch ? 0u : 256u;
   a.perm = nullptr;
-  a.flat = group == 1 ? 1u : 0u;
   int sms = 1;
   SZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ix->device));
-  a.NP = nw;
-  nw = search_warps(group, p->cta_warps, nq, (uint32_t)sms);
-  size_t smem = search_layout(a, nw);
-  if (smem > 200 * 1024 && !p->cta_warps) smem = search_layout(a, nw = 8);
-  if (smem > 200 * 1024) return fail(SEISMIC_EBUDGET, "search: shared memory per query exceeds 200 KB");
+  const size_t smem = search_fit(a, group, p->cta_warps, (uint32_t)sms, 0u, nw);
+  if (smem == 0) return fail(SEISMIC_EBUDGET, "search: shared memory per query exceeds 200 KB");
   int blocks = 1;
   if ((rc = search_occupancy(group, nw, smem, &blocks))) return rc;
   uint64_t grid = std::min<uint64_t>(nq, (uint64_t)std::max(1, blocks) * sms);

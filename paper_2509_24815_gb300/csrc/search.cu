@@ -443,13 +443,14 @@ __device__ __forceinline__ void eval_wave_flat(const SearchArgs &a, Smem &s, Sha
   uint32_t *queue = reinterpret_cast<uint32_t *>(s.wqueue() + warp * kWarpQueueBytes);
   float2 *sums = reinterpret_cast<float2 *>(queue);
   const uint8_t *qf = s.qfilt();
-  const uint32_t dpw = min(32u, (n + NW - 1) / NW);
+  const uint32_t per = (n + NW - 1) / NW, rounds = (per + 31u) / 32u, dpw = (per + rounds - 1) / rounds;
   const bool crowded = sh.hash_n > a.HS / 4 * 3;
-  for (uint32_t r0 = 0; r0 < n; r0 += NW * 32) {  // one round, unless n > 32 NW
-    const uint32_t i = r0 + warp * dpw + lane;
+  const uint32_t mine = min(n, (warp + 1) * per);  // the warp's members: warp * per .. mine
+  for (uint32_t r0 = warp * per; r0 < mine; r0 += dpw) {
+    const uint32_t i = r0 + lane;
     uint32_t d = SEISMIC_NONE_ID, nch = 0;
     unsigned long long row = 0ull;
-    if (lane < dpw && i < n) {
+    if (lane < dpw && i < mine) {
       src.fetch(i, d, row);
       bool fresh = false;
       if (d != SEISMIC_NONE_ID) {
@@ -529,15 +530,21 @@ __device__ __forceinline__ void eval_wave_flat(const SearchArgs &a, Smem &s, Sha
           v = ldg_na_f32(wd.val[x] + 4u * pos);
         }
         const uint32_t hits = __ballot_sync(0xffffffffu, hit);
-        const uint32_t later = lane < 31u ? firsts & (~0u << (lane + 1u)) : 0u;
-        const uint32_t len = (firsts >> lane) & 1u ? (later ? __ffs(later) - 1u : cnt) - lane : 0u;  // a first entry's chunk
-        const uint32_t longest = __reduce_max_sync(0xffffffffu, len);
         float acc = hit ? fmaf(q, v, 0.0f) : 0.0f;
-        for (uint32_t o = 1; o < longest; o++) {
-          const float q2 = __shfl_down_sync(0xffffffffu, q, o), v2 = __shfl_down_sync(0xffffffffu, v, o);
-          if (o < len && ((hits >> (lane + o)) & 1u)) acc = fmaf(q2, v2, acc);
+        // hits behind another one of their chunk: chained in entry order onto the chunk's first entry
+        const uint32_t self = firsts & (below | (1u << lane)), run = self ? 31u - __clz(self) : 0u;
+        const bool again = hit && (hits & below & (~0u << run));
+        if (__any_sync(0xffffffffu, again)) {
+          const uint32_t later = lane < 31u ? firsts & (~0u << (lane + 1u)) : 0u;
+          const uint32_t len = (firsts >> lane) & 1u ? (later ? __ffs(later) - 1u : cnt) - lane : 0u;  // a first entry's chunk
+          const uint32_t longest = __reduce_max_sync(0xffffffffu, len);
+          for (uint32_t o = 1; o < longest; o++) {
+            const float q2 = __shfl_down_sync(0xffffffffu, q, o), v2 = __shfl_down_sync(0xffffffffu, v, o);
+            if (o < len && ((hits >> (lane + o)) & 1u)) acc = fmaf(q2, v2, acc);
+          }
+          if (len == 0) acc = 0.0f;
         }
-        if (lane < cnt) queue[r + lane] = len ? __float_as_uint(acc) : 0u;
+        if (lane < cnt) queue[r + lane] = __float_as_uint(acc);
         r += cnt;
       }
       __syncwarp();
@@ -785,7 +792,9 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
     }
     __syncthreads();
     // ---------------------------------------------------------- H1: list terms
-    if (a.alpha_q > 0.0f) {
+    if (a.seed) {
+      if (tid == 0) sh.ncut = 0;  // graph refinement: no lists
+    } else if (a.alpha_q > 0.0f) {
       for (uint32_t i = tid; i < nzq; i += NT) {
         const float av = fabsf(s.qval()[i]);
         const uint32_t t = s.qterm()[i];
@@ -825,7 +834,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
       if (tid == 0) sh.ncut = min(cut, nzq);
     }
     __syncthreads();
-    const uint32_t ncut = a.seed ? 0u : sh.ncut;  // graph refinement: no lists
+    const uint32_t ncut = sh.ncut;
     const float hf = sh.hf;
     if (a.stats && tid == 0) sh.st[SEISMIC_ST_QUERY_NNZ] = nnz;
 
@@ -895,7 +904,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
       // ---- H3: order blocks by (r desc, block asc)
       bitonic_sort_u64<NT>(s.keys(), P2);
       // ---- H4/H5/H6: visit blocks in order.  A wave is the next W blocks that
-      // pass the test against theta (fewer past CAND documents; a larger block
+      // pass the test against theta (fewer past kCand documents; a larger block
       // goes alone, in pieces).  Group 1 scores as many whole waves at once as
       // fit CAND documents, as if theta stayed; when it rose so far that a later
       // wave would have tested otherwise, the waves are merged one by one and
@@ -912,7 +921,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
         nd = 0;
         while (e < last && e - p < W) {
           const uint32_t b = (uint32_t)(keys[e] & 0xFFFFFFFFu), bn = s.bptr()[b + 1] - s.bptr()[b];
-          if (e > p && ((full && bscore(e) < thr) || nd + bn > a.CAND)) break;
+          if (e > p && ((full && bscore(e) < thr) || nd + bn > kCand)) break;
           nd += bn;
           e++;
         }
@@ -1025,7 +1034,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
 template <int G, int NW>
 int launch_t(const SearchArgs &a, size_t smem, uint32_t grid, cudaStream_t st) {
   static std::atomic<uint64_t> configured{0};
-  int rc = set_smem_limit_once(configured, (const void *)k_search<G, NW>, 200 * 1024);
+  int rc = set_smem_limit_once(configured, (const void *)k_search<G, NW>, (int)kMaxSmem);
   if (rc) return rc;
   k_search<G, NW><<<grid, NW * 32, smem, st>>>(a);
   SZ_CUDA(cudaGetLastError());
@@ -1034,7 +1043,7 @@ int launch_t(const SearchArgs &a, size_t smem, uint32_t grid, cudaStream_t st) {
 
 template <int G, int NW>
 int occupancy_t(size_t smem, int *blocks) {
-  SZ_CUDA(cudaFuncSetAttribute(k_search<G, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  SZ_CUDA(cudaFuncSetAttribute(k_search<G, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
   SZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_search<G, NW>, NW * 32, smem));
   return SEISMIC_OK;
 }
@@ -1056,7 +1065,6 @@ size_t search_layout(SearchArgs &a, uint32_t nw) {
   a.off_qterm = take(a.QN * 2);
   a.off_cut = take(a.QN * 2);
   a.off_aq = take(a.alpha_q > 0.0f ? a.QN * 4 : 4);
-  if (!a.NP) a.NP = nw;
   a.off_part = take(a.exhaustive ? 4 : a.NP * a.BMAX * 4);
   a.off_keys = take(a.exhaustive ? 8 : a.BPOW2 * 8);
   const uint32_t nclo = std::max(a.QN, a.k);  // clo also holds S during the expansion
@@ -1073,6 +1081,11 @@ size_t search_layout(SearchArgs &a, uint32_t nw) {
   a.off_cand_i = take(a.flat ? a.CAND * 2 : 0);
   a.off_fresh = take(a.flat ? a.CAND : 0);
   a.off_bptr = take(a.exhaustive ? 4 : (a.BMAX + 1) * 4);
+  // what a call is refused by (search_fit): the query's data, a wave's candidates (9 bytes each) and, for group 1,
+  // 3 KB and a byte per block-score entry, 2048 entries at least
+  const uint32_t entries = a.exhaustive ? 0u : nw * a.BMAX;
+  a.budget = o;
+  if (a.flat) a.budget += kCand * 9u + 3088u + std::max(2048u, entries) + (entries < 2048u ? 8192u : 0u) - a.CAND * 12u;
   if (a.flat) {
     // the warps' candidate queues: in the block-score partials' space (dead
     // while documents are scored) where they fit
@@ -1086,13 +1099,40 @@ size_t search_layout(SearchArgs &a, uint32_t nw) {
 
 // A query alone on its SM is bound by latency: the more warps share a wave's
 // documents, the fewer loads follow one another.  One CTA of 32 warps per SM up
-// to as many queries as SMs, 16 warps up to twice that, else 8 (one query, 1M documents, cut 10: 3.0 ms with 8 warps, 2.4 with
-// 32; 1000 queries, 100k documents: 2.6 ms with 8, 3.2 with 16).
-// The block scores are added up as by 8 warps in each (SearchArgs::NP), so the
-// results do not depend on the choice.
-uint32_t search_warps(uint32_t group, uint32_t asked, uint32_t nq, uint32_t sms) {
-  if (asked) return asked;
-  return group != 1 || nq > 2 * sms ? 8u : nq > sms ? 16u : 32u;
+// to as many queries as SMs, 16 warps up to twice that, else 8 (one query, 1M
+// documents, cut 10: 3.0 ms with 8 warps, 2.4 with 32; 1000 queries, 100k documents:
+// 2.6 ms with 8, 3.2 with 16).  The block scores are added up as by 8 warps in
+// each (SearchArgs::NP), so the results do not depend on the choice.
+static uint32_t search_warps(uint32_t nq, uint32_t sms) { return nq > 2 * sms ? 8u : nq > sms ? 16u : 32u; }
+
+size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t sms, uint32_t bitmap_words, uint32_t &nw) {
+  nw = asked ? asked : 8u;
+  a.NP = nw;
+  a.flat = group == 1 ? 1u : 0u;
+  a.CAND = kCand;
+  size_t smem = search_layout(a, nw);
+  if (a.budget > 200u * 1024u) return 0;
+  if (a.persistent) a.HS = 16;  // the seen set is a bitmap in global memory
+  if (!a.flat) return search_layout(a, nw);
+  const uint32_t slots = a.HS, wide = asked ? asked : search_warps(a.nq, sms);
+  for (int form = bitmap_words ? 0 : 1; form < 2; form++) {
+    a.seen_words = form == 0 ? bitmap_words : 0u;
+    a.HS = form == 0 ? bitmap_words : slots;
+    for (uint32_t w : {wide, nw}) {
+      // wide CTAs score more documents at once: one query 1.45 ms instead of 1.77, but batches of 8-warp
+      // CTAs 65.9 instead of 63.7
+      a.CAND = w > nw ? kWideCand : kCand;
+      if ((smem = search_layout(a, w)) <= kMaxSmem) {
+        nw = w;
+        return smem;
+      }
+    }
+  }
+  // very long queries: the lane groups need less besides the query
+  group = 8;
+  a.flat = 0;
+  a.CAND = kCand;
+  return search_layout(a, nw);
 }
 
 int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, uint32_t grid, cudaStream_t st) {

@@ -64,14 +64,16 @@ struct SearchArgs {
   uint32_t flat;
   // shared-memory layout
   uint32_t W, QN, BMAX, BPOW2, HS, CAND;
-  uint32_t NP;  // block-score partial arrays, one per warp that scores summaries (0: the CTA's warps)
+  uint32_t NP;      // block-score partial arrays, one per warp that scores summaries
+  uint32_t budget;  // bytes that count towards the limit on a query's shared memory
   uint32_t off_qbits, off_qrank, off_qval, off_qterm, off_cut, off_aq, off_part, off_keys, off_clo, off_chi,
       off_hash, off_tk_s, off_tk_id, off_tmp_s, off_tmp_id, off_cand_s, off_cand_id, off_cand_ok,
       off_wdocs, off_wqueue, off_qfilt, off_cand_i, off_fresh, off_bptr;
 };
 
 // CTA kernel, group 1
-constexpr uint32_t kCand = 256;          // documents scored at once (SearchArgs::CAND)
+constexpr uint32_t kCand = 256;          // documents of a wave at most (but for a larger block)
+constexpr uint32_t kWideCand = 512;      // documents scored at once (SearchArgs::CAND) by more than 8 warps of their own choice
 constexpr uint32_t kSeenDocs = 131072;   // collections up to here keep a launch's seen set as a bitmap in shared memory
 constexpr uint32_t kFilter = 8192;        // bytes of the query's term filter
 constexpr uint32_t kWarpQueueBytes = 1536;  // a warp's candidate queue
@@ -80,8 +82,12 @@ constexpr uint32_t kShortChunks = 256;    // chunks of a row whose positions fit
 constexpr uint32_t kMaxWave = 64;  // blocks per wave (CTA kernel)
 size_t search_layout(SearchArgs &a, uint32_t nw);
 int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, uint32_t grid, cudaStream_t st);
-// The warps per CTA of a search of nq queries that leaves them open (0).
-uint32_t search_warps(uint32_t group, uint32_t asked, uint32_t nq, uint32_t sms);
+constexpr uint32_t kMaxSmem = 226u * 1024u;  // dynamic shared memory of a CTA, beside a little static
+// Chooses warps per CTA (asked, or by the number of queries), the seen set
+// (bitmap_words > 0: a bitmap in shared memory where it fits) and, for queries
+// too long for group 1's arrays, lane groups; lays shared memory out and
+// returns its size, or 0 when the query's data exceed 200 KB.
+size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t sms, uint32_t bitmap_words, uint32_t &nw);
 int search_occupancy(uint32_t group, uint32_t nw, size_t smem, int *blocks);
 size_t search_layout_warp(SearchArgs &a);
 int launch_search_warp(const SearchArgs &a, uint32_t group, size_t smem, uint32_t grid, uint32_t wpb,

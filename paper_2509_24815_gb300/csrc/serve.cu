@@ -238,12 +238,13 @@ int seismic_server_create(seismic_index *ix, const seismic_search_params *search
       a.BPOW2 = 1;
       while (a.BPOW2 < a.BMAX) a.BPOW2 <<= 1;
       a.HS = 16;
-      a.CAND = kCand;
       a.k = std::max<uint32_t>(search->k, 100);
       a.alpha_q = search->alpha_q;
       const uint32_t nw = search->cta_warps ? search->cta_warps : 8, g = search->group ? search->group : 1;
       a.dim = ix->dim;
       a.flat = g == 1 ? 1u : 0u;
+      a.CAND = kCand;
+      a.NP = nw;
       size_t smem = search_layout(a, nw);
       int blocks = 1;
       int rc = search_occupancy(g, nw, smem, &blocks);
