@@ -19,7 +19,7 @@ import numpy as np
 from . import DeviceCSR, search_params, seismic_info, seismic_search
 
 # (shape, group, cta_warps, wave, L2 row prefetch): shape 1 = one CTA per query
-# (group 1: chunk-flattened scoring, else lane groups of that width), 2 = one
+# (group 1: warp-local scoring, else lane groups of that width), 2 = one
 # warp per query
 DEFAULT_CANDIDATES = tuple(
     [(1, 1, 8, v, pf) for v in (4, 8, 16, 32) for pf in (False, True)] +

@@ -129,7 +129,7 @@ extern "C" int seismic_search_noalloc(seismic_index *ix, const seismic_csr *quer
   a.perm = nullptr;
   int sms = 1;
   SZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ix->device));
-  const size_t smem = search_fit(a, group, p->cta_warps, (uint32_t)sms, 0u, nw);
+  const size_t smem = search_fit(a, group, p->cta_warps, 0u, (uint32_t)sms, 0u, nw);
   if (smem == 0) return fail(SEISMIC_EBUDGET, "search: shared memory per query exceeds 200 KB");
   int blocks = 1;
   if ((rc = search_occupancy(group, nw, smem, &blocks))) return rc;

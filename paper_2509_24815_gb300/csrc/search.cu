@@ -1105,7 +1105,8 @@ size_t search_layout(SearchArgs &a, uint32_t nw) {
 // each (SearchArgs::NP), so the results do not depend on the choice.
 static uint32_t search_warps(uint32_t nq, uint32_t sms) { return nq > 2 * sms ? 8u : nq > sms ? 16u : 32u; }
 
-size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t sms, uint32_t bitmap_words, uint32_t &nw) {
+size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefer, uint32_t sms, uint32_t bitmap_words,
+                  uint32_t &nw) {
   nw = asked ? asked : 8u;
   a.NP = nw;
   a.flat = group == 1 ? 1u : 0u;
@@ -1114,7 +1115,7 @@ size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t sms, 
   if (a.budget > 200u * 1024u) return 0;
   if (a.persistent) a.HS = 16;  // the seen set is a bitmap in global memory
   if (!a.flat) return search_layout(a, nw);
-  const uint32_t slots = a.HS, wide = asked ? asked : search_warps(a.nq, sms);
+  const uint32_t slots = a.HS, wide = asked ? asked : prefer ? prefer : search_warps(a.nq, sms);
   for (int form = bitmap_words ? 0 : 1; form < 2; form++) {
     a.seen_words = form == 0 ? bitmap_words : 0u;
     a.HS = form == 0 ? bitmap_words : slots;
