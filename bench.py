@@ -62,11 +62,10 @@ RECALL_TARGET = 0.9
 K = 10
 METRIC = "QPS at recall@10>=0.9 (batched Seismic search, fixed parameters)"
 # DRAM traffic of k_search per byte it executes (read + write), from one ncu capture of the current
-# kernel on the 300k-document workload (fp32 rows, wave 8), keyed by the L2 row prefetch (which
-# brings whole rows in); used to estimate a full launch's traffic from its executed bytes.  A form
-# without a capture of the current kernel reports null.
-TRAFFIC_PER_EXEC_BYTE = {False: (14.940076544e9 + 0.615757056e9) / 24.652337535e9,
-                         True: (19.571495424e9 + 0.855928576e9) / 24.652337535e9}
+# kernel on 300k documents (fp32 rows, cut 10, heap_factor 0.8, wave 8), keyed by the L2 prefetch (of
+# member lists; rows are read in units where they are needed); used to estimate a full launch's traffic
+# from its executed bytes.  A form without a capture of the current kernel reports null.
+TRAFFIC_PER_EXEC_BYTE = {True: (16.156699e9 + 0.916050e9) / 41.034674e9}
 
 
 def log(*a):
@@ -415,7 +414,7 @@ def main():
     ap.add_argument("--workload", default=DEFAULT_WORKLOAD, choices=sorted(WORKLOADS))
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--group", type=int, default=1, help="1: chunk-flattened scoring, 8/16/32: lane groups")
+    ap.add_argument("--group", type=int, default=1, help="1: warp-local scoring, 8/16/32: lane groups")
     ap.add_argument("--cta-warps", type=int, default=0)
     ap.add_argument("--wave", type=int, default=16)
     ap.add_argument("--persistent", type=int, default=1)
