@@ -2,7 +2,7 @@
 // judge, and the exact kappa-NN graph (Eq. "knn-graph") for small
 // collections.
 //
-// The collection is cut into tiles of up to kExTile documents whose fp32
+// The collection is cut into tiles of up to ex_tile documents whose fp32
 // accumulators fit shared memory.  A CTA takes a query (or, when there are
 // fewer queries than CTAs, a share of its tiles) and, tile by tile, adds the
 // query's terms in ascending order: the postings of a term inside the tile are
@@ -26,8 +26,13 @@ namespace seismic {
 namespace {
 
 constexpr uint32_t kExNT = 512;
-constexpr uint32_t kExTile = 16384;    // documents of a tile: 64 KB of accumulators, three CTAs per SM
-constexpr uint32_t kExSplitCtas = 3;   // CTAs per SM below which queries are split
+// Two CTAs per SM: 64 registers per thread, and tiles as large as leave room for two beside the sort area (k <= 256:
+// 24,576 documents, 96 KB; more: 16,384 and a sort area four times as large).  1000 queries of 10..150 entries, 1M
+// documents: 10.3 ms; with 16,384 documents 13.7, with three CTAs (40 registers, 14,848 documents) 11.4.
+constexpr uint32_t kExCtas = 2;
+constexpr uint32_t ex_area(uint32_t k) { return k <= 256u ? 1024u : 4096u; }
+constexpr uint32_t ex_tile(uint32_t k) { return k <= 256u ? 24576u : 16384u; }
+constexpr size_t ex_smem(uint32_t k, uint32_t tile) { return (size_t)ex_area(k) * 8 + (size_t)k * 8 + (size_t)tile * 4; }
 
 __device__ __forceinline__ uint32_t f2ord(float f) {
   uint32_t u = __float_as_uint(f);
@@ -43,6 +48,8 @@ __device__ __forceinline__ unsigned long long mkkey(float s, uint32_t id) {
 }
 
 constexpr uint32_t kExGroups = 1024;  // group maxima that bound a first tile's k-th best; at least kExactMaxK
+constexpr size_t kExSmem = std::max(ex_smem(256, ex_tile(256)), ex_smem(kExactMaxK, ex_tile(kExactMaxK)));
+static_assert(kExCtas * (kExSmem + 7u * 1024u + 1024u) <= 228u * 1024u, "two CTAs, their ExShared and what each reserves");
 static_assert(kExGroups >= kExactMaxK && kExGroups % kExNT == 0, "a group maximum per result, whole groups per thread");
 
 struct ExShared {
@@ -116,7 +123,7 @@ __global__ void __launch_bounds__(kExNT) k_exact_bounds(const ExactArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(kExNT) k_exact(const ExactArgs a) {
+__global__ void __launch_bounds__(kExNT, kExCtas) k_exact(const ExactArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ ExShared sh;
   unsigned long long *cb = reinterpret_cast<unsigned long long *>(sm);  // sort area: buffer + top-k
@@ -252,28 +259,28 @@ __global__ void __launch_bounds__(kExNT) k_exact_join(const ExactArgs a) {
 // Working memory: the bounds table, the claim words and the splits' results; it
 // depends on the index only, so it is allocated once.
 size_t exact_layout(ExactArgs &a, uint32_t sms, void *base) {
-  a.tiles = (a.n_docs + kExTile - 1) / kExTile;
+  a.tiles = (a.n_docs + ex_tile(a.k) - 1) / ex_tile(a.k);
   a.tile = (a.n_docs + a.tiles - 1) / a.tiles;
-  a.area = a.k <= 256 ? 1024u : 4096u;
+  a.area = ex_area(a.k);
   a.sms = sms;
   const size_t claim = ((size_t)a.dim * 4 + 255) & ~(size_t)255;
-  const size_t bounds = ((size_t)a.dim * (a.tiles + 1) * 4 + 255) & ~(size_t)255;
+  const uint32_t most = (a.n_docs + ex_tile(kExactMaxK) - 1) / ex_tile(kExactMaxK);
+  const size_t bounds = ((size_t)a.dim * (most + 1) * 4 + 255) & ~(size_t)255;
   unsigned char *p = reinterpret_cast<unsigned char *>(base);
   a.claim = reinterpret_cast<uint32_t *>(p);
   a.bounds = reinterpret_cast<uint32_t *>(p + claim);
   a.part = reinterpret_cast<unsigned long long *>(p + claim + bounds);
-  return claim + bounds + (size_t)2 * kExSplitCtas * sms * kExactMaxK * 8;
+  return claim + bounds + (size_t)kExCtas * sms * kExactMaxK * 8;
 }
 
 int launch_exact(ExactArgs a, cudaStream_t st) {
   if (a.k == 0 || a.k > kExactMaxK) return fail(SEISMIC_EINVAL, "exact search: k must be in 1..1024");
-  // fewer queries than CTAs that run at once: several CTAs share a query's tiles
-  const uint32_t ctas = kExSplitCtas * a.sms;
-  a.splits = a.nq >= ctas ? 1u : std::min(a.tiles, (ctas + a.nq - 1) / a.nq);
-  const size_t smem = (size_t)a.area * 8 + (size_t)a.k * 8 + (size_t)a.tile * 4;
+  // fewer queries than CTAs that run at once: several CTAs share a query's tiles, as many as all run at once
+  a.splits = std::max(1u, std::min(a.tiles, kExCtas * a.sms / a.nq));
+  const size_t smem = ex_smem(a.k, a.tile);
   static std::atomic<uint64_t> configured{0}, configured2{0};
   int rc;
-  if ((rc = set_smem_limit_once(configured, (const void *)k_exact, (int)(4096 * 8 + kExactMaxK * 8 + kExTile * 4))) ||
+  if ((rc = set_smem_limit_once(configured, (const void *)k_exact, (int)kExSmem)) ||
       (rc = set_smem_limit_once(configured2, (const void *)k_exact_join, (int)(4096 * 8 + kExactMaxK * 8))))
     return rc;
   SZ_CUDA(cudaMemsetAsync(a.claim, 0, (size_t)a.dim * 4, st));

@@ -1,0 +1,45 @@
+"""Calls at the sizes where a kernel takes another route: each against an exact reference computed here, or against
+the route that the same call takes under other launch parameters."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _rows(n, terms_of, vlo, vhi, dim, rng):
+    """n sparse rows of small whole values (fp32 sums of products are exact, and ties are common); terms_of(i) gives
+    row i's terms."""
+    t = [np.unique(terms_of(i)) for i in range(n)]
+    indptr = np.zeros(n + 1, dtype=np.uint64)
+    np.cumsum([len(x) for x in t], out=indptr[1:])
+    vals = rng.integers(vlo, vhi + 1, int(indptr[-1]))
+    vals[vals == 0] = 1
+    return synth.CSR(indptr, np.concatenate(t).astype(np.uint16), vals.astype(np.float32), dim)
+
+
+def _scores(queries, docs):
+    sp = pytest.importorskip("scipy.sparse")
+
+    def csr(m):
+        return sp.csr_matrix((m.vals.astype(np.float64), m.terms.astype(np.int64), m.indptr.astype(np.int64)),
+                             shape=(m.n_rows, m.dim))
+    return (csr(queries) @ csr(docs).T).toarray()
+
+
+# Exact search: tiles of 24,576 documents up to k = 256, of 16,384 past it, and as many CTAs per query as run at once.
+@pytest.mark.parametrize("n_docs", [24576, 24577, 49153])
+@pytest.mark.parametrize("nq,k", [(1, 256), (1, 257), (150, 10), (310, 256)])
+def test_exact_search_tile_edges(sz, n_docs, nq, k):
+    dim = 61
+    rng = np.random.default_rng(n_docs + k)
+    docs = _rows(n_docs, lambda i: rng.integers(0, dim, rng.integers(1, 6)), -2, 5, dim, rng)
+    queries = _rows(nq, lambda i: rng.integers(0, dim, rng.integers(1, 40)), -1, 3, dim, rng)
+    ix = sz.seismic_build(docs, lambda_=10, beta=2, alpha=0.5, seed=1, keep_full_lists=True)
+    ids, sc = sz.seismic_search_exact(ix, queries, k)
+    ix.close()
+    score = _scores(queries, docs)
+    order = np.argsort(-score, axis=1, kind="stable")[:, :k]  # score descending, id ascending
+    np.testing.assert_array_equal(ids, order.astype(np.uint32))
+    np.testing.assert_array_equal(sc, np.take_along_axis(score, order, 1).astype(np.float32))
