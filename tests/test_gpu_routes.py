@@ -43,3 +43,24 @@ def test_exact_search_tile_edges(sz, n_docs, nq, k):
     order = np.argsort(-score, axis=1, kind="stable")[:, :k]  # score descending, id ascending
     np.testing.assert_array_equal(ids, order.astype(np.uint32))
     np.testing.assert_array_equal(sc, np.take_along_axis(score, order, 1).astype(np.float32))
+
+
+# Exact search: a tile (24,576 documents, 16,384 past k = 256) without a posting of the query is passed over and one
+# with few of them offers only those, once documents of score 0 cannot enter any more.  Queries of one rare term, of
+# some (their offers wait over several tiles) and of many and common ones; negative scores, which rank behind 0.
+@pytest.mark.parametrize("n_docs", [24577, 70003])
+@pytest.mark.parametrize("nq,k", [(1, 1), (3, 10), (400, 10), (400, 256), (700, 3), (40, 257), (400, 1000)])
+def test_exact_search_of_rare_terms(sz, n_docs, nq, k):
+    dim = 3000
+    rng = np.random.default_rng(n_docs + k)
+    docs = _rows(n_docs, lambda i: np.concatenate([rng.integers(0, 4, 1), rng.integers(4, dim, rng.integers(1, 4))]), -2, 5,
+                 dim, rng)
+    sizes = [1, 1, 2, 7, 25, 60, 600]
+    queries = _rows(nq, lambda i: rng.integers(4 if i % 5 else 0, dim, sizes[i % 7]), -1 if nq > 1 else 1, 3, dim, rng)
+    ix = sz.seismic_build(docs, lambda_=10, beta=2, alpha=0.5, seed=1, keep_full_lists=True)
+    ids, sc = sz.seismic_search_exact(ix, queries, k)
+    ix.close()
+    score = _scores(queries, docs)
+    order = np.argsort(-score, axis=1, kind="stable")[:, :k]  # score descending, id ascending
+    np.testing.assert_array_equal(ids, order.astype(np.uint32))
+    np.testing.assert_array_equal(sc, np.take_along_axis(score, order, 1).astype(np.float32))
