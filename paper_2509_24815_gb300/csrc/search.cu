@@ -946,7 +946,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
           ndocs += nd;
           be = e;
         }
-        if (a.prefetch && tid < max(W, 8u) && be + tid < nb) {  // member lists of the next blocks
+        if (a.prefetch && tid < (G == 1 ? max(W, 8u) : W) && be + tid < nb) {  // member lists of the next blocks
           const uint32_t b = (uint32_t)(keys[be + tid] & 0xFFFFFFFFu);
           const uint32_t e0 = s.bptr()[b], e1 = s.bptr()[b + 1];
           prefetch_l2(a.bdoc + e0, 4 * (e1 - e0));
@@ -954,11 +954,14 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
         }
         uint32_t done = be, taken = ndocs;  // blocks up to here, and their documents, count
         for (uint32_t c0 = 0; c0 < ndocs; c0 += a.CAND) {  // one round, unless a single block is larger
-          const ListSrc src{keys + bi, s.bptr(), be - bi, c0, a.bdoc, a.bdoc_row};
+          // (lane groups: one block's members lie side by side, no walk over the blocks' sizes)
+          const bool single = G != 1 && be - bi == 1;
+          const ListSrc src{keys + bi, s.bptr(), single ? 0u : be - bi,
+                            single ? s.bptr()[(uint32_t)(keys[bi] & 0xFFFFFFFFu)] + c0 : c0, a.bdoc, a.bdoc_row};
           const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, ndocs - c0), src, 0);
           if (m == 0) continue;
           const uint32_t nc = merge_rank<NT>(a, s, sh, m, false, 0, 0);
-          if (be == first_end || nc < a.k || bscore(be - 1) >= limit(s.tmp_s()[a.k - 1])) {
+          if (G != 1 || be == first_end || nc < a.k || bscore(be - 1) >= limit(s.tmp_s()[a.k - 1])) {
             merge_commit<NT>(s, sh, nc, true);
             continue;
           }

@@ -39,13 +39,14 @@ __device__ __forceinline__ float qlookup(const uint32_t *__restrict__ qbits, con
 }
 
 // Read-only loads that do not allocate in L1 (rows are read once per query;
-// reuse across queries is in L2) and fetch 64 bytes, not a whole 128-byte line,
-// from DRAM on a miss: a scattered 32-byte read moved 124 bytes from DRAM
-// without the L2::64B qualifier and 63 with it (3 GB buffer).  ldg_na reads 16
-// bytes, ldg_na_v8 32 bytes (one sector; p is 32-byte aligned), ldg_na_f32 one float.
+// reuse across queries is in L2).  ldg_na reads 16 bytes, ldg_na_v8 32 bytes (one
+// sector; p is 32-byte aligned), ldg_na_f32 one float.  The latter two, of rows
+// that nobody has prefetched, fetch 64 bytes, not a whole 128-byte line, from
+// DRAM on a miss: a scattered 32-byte read moved 124 bytes from DRAM without the
+// L2::64B qualifier and 63 with it (3 GB buffer).
 __device__ __forceinline__ uint4 ldg_na(const void *p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;
