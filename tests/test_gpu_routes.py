@@ -64,3 +64,41 @@ def test_exact_search_of_rare_terms(sz, n_docs, nq, k):
     order = np.argsort(-score, axis=1, kind="stable")[:, :k]  # score descending, id ascending
     np.testing.assert_array_equal(ids, order.astype(np.uint32))
     np.testing.assert_array_equal(sc, np.take_along_axis(score, order, 1).astype(np.float32))
+
+
+@pytest.fixture(scope="module", params=[False, True], ids=["fp32", "fp16"])
+def collection(sz, request):
+    """3000 rows of 1..60 of 300 terms, some of them longer than a queue's positions, and a graph."""
+    dim = 4000
+    rng = np.random.default_rng(3)
+    docs = _rows(3000, lambda i: rng.integers(0, dim, 3500) if i % 500 == 7 else rng.integers(0, 300, rng.integers(1, 61)),
+                 -1, 4, dim, rng)
+    queries = _rows(1400, lambda i: rng.integers(0, 320, rng.integers(1, 90)), -1, 3, dim, rng)
+    ix = sz.seismic_build(docs, lambda_=300, beta=40, alpha=0.6, quantize_u8=False, seed=2, values_fp16=request.param)
+    sz.seismic_set_knn(ix, rng.integers(0, docs.n_rows, (docs.n_rows, 5)))
+    yield queries, ix
+    ix.close()
+
+
+# The default launch (group 1) by the number of queries: CTAs of 32, 16 and 8 warps, five CTAs of 8 warps per SM;
+# waves are scored together from the first full top-k on.  Lane groups score one row and one wave at a time; sums of
+# whole values are exact in any order, so the documents, the scores and the work counted have to be the same.
+@pytest.mark.parametrize("kw", [dict(wave=1), dict(wave=1, k=70, heap_factor=1.0), dict(wave=8, k=100), dict(wave=8, use_knn=True),
+                                dict(wave=3, hf_mode=1, heap_factor=0.9), dict(exhaustive=True), dict(wave=2, cta_warps=8)],
+                         ids=lambda d: ",".join(f"{k}={v}" for k, v in d.items()))
+@pytest.mark.parametrize("launch", [dict(persistent=True), dict(persistent=False), dict(persistent=False, hash_slots=32)],
+                         ids=["persistent", "plain", "tiny hash"])
+@pytest.mark.parametrize("nq", [2, 200, 500, 700, 1400])
+def test_default_launch_by_number_of_queries(sz, collection, kw, launch, nq):
+    queries, ix = collection
+    q = queries.slice(0, nq)
+    kw = dict(dict(k=10, cut=8, heap_factor=0.8), **kw)
+    gi, gs, gst = sz.seismic_search(ix, q, stats=True, **launch, **kw)
+    ri, rs, rst = sz.seismic_search(ix, q, group=32, persistent=True, stats=True, **dict(kw, cta_warps=8))
+    np.testing.assert_array_equal(gs, rs)
+    np.testing.assert_array_equal(gi, ri)
+    for name in ("lists", "blocks_scored", "blocks_evaluated", "blocks_skipped", "block_docs", "summary_entries"):
+        np.testing.assert_array_equal(gst[:, sz.STATS.index(name)], rst[:, sz.STATS.index(name)], err_msg=name)
+    if "hash_slots" not in launch:  # a set that forgets scores some documents again
+        for name in ("docs", "doc_nnz", "knn_docs", "knn_nnz"):
+            np.testing.assert_array_equal(gst[:, sz.STATS.index(name)], rst[:, sz.STATS.index(name)], err_msg=name)
