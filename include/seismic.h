@@ -107,8 +107,9 @@ typedef struct {
                             that width score one row each.  Warp shape: 4/8/16/32 lanes per
                             row.  0 = 1 on the CTA shape, 8 on the warp shape.  Scores differ
                             only in fp32 summation order */
-  uint32_t cta_warps;    /* warps per CTA: 4, 8 or 16; 0 = 8, or more with group 1 and fewer queries
-                            than the GPU holds (the results are those of 8) */
+  uint32_t cta_warps;    /* warps per CTA: 4, 8 or 16; 0 = 8, or with group 1 up to four queries per
+                            SM 16 or 32 (the results are those of 8).  With group 1, queries too
+                            long for its shared memory go by lane groups of 8 */
   uint32_t persistent;   /* 1: one persistent launch that pulls queries from a device queue */
   uint32_t max_query_nnz; /* device queries: an upper bound on any query's nonzeros, which sizes
                             shared memory; 0 = measure it (one device synchronisation, so not

@@ -1113,11 +1113,12 @@ static size_t search_budget(const SearchArgs &a, uint32_t nw) {
 
 // A query alone on its SM is bound by latency: the more warps share a wave's
 // documents, the fewer loads follow one another.  One CTA of 32 warps per SM up
-// to as many queries as SMs, 16 warps up to twice that, else 8 (one query, 1M
-// documents, cut 10: 3.0 ms with 8 warps, 2.4 with 32; 1000 queries, 100k documents:
-// 2.6 ms with 8, 3.2 with 16).  The block scores are added up as by 8 warps in
-// each (SearchArgs::NP), so the results do not depend on the choice.
-static uint32_t search_warps(uint32_t nq, uint32_t sms) { return nq > 2 * sms ? 8u : nq > sms ? 16u : 32u; }
+// to as many queries as SMs, 16 warps up to four times that (two CTAs per SM, in
+// up to two rounds), else 8.  1M documents, cut 10: one query 2.6 ms with 8 warps,
+// 1.5 with 32; 305 queries 4.95 with 8, 3.35 with 16; 450: 6.2, 5.2; 608: 6.6, 6.2; 700: 6.9,
+// 7.6.  The block scores are added up as by 8 warps in each (SearchArgs::NP), so the results do
+// not depend on the choice.
+static uint32_t search_warps(uint32_t nq, uint32_t sms) { return nq > 4 * sms ? 8u : nq > sms ? 16u : 32u; }
 
 size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefer, uint32_t sms, uint32_t bitmap_words,
                   uint32_t &nw) {
