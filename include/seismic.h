@@ -103,8 +103,8 @@ typedef struct {
   uint32_t group;        /* how documents are scored.  CTA shape: 1 = each warp goes over the rows
                             of its share of the wave laid end to end (seen documents are dropped
                             before their rows are read; small waves are scored together, with the
-                            results and counters of one after the other), 8/16/32 = lane groups of
-                            that width score one row each.  Warp shape: 4/8/16/32 lanes per
+                            results of one after the other, and its counters where the seen set is
+                            a bitmap), 8/16/32 = lane groups of that width score one row each.  Warp shape: 4/8/16/32 lanes per
                             row.  0 = 1 on the CTA shape, 8 on the warp shape.  Scores differ
                             only in fp32 summation order */
   uint32_t cta_warps;    /* warps per CTA: 4, 8 or 16; 0 = 8, or with group 1 up to four queries per
@@ -116,8 +116,8 @@ typedef struct {
                             inside stream capture).  Ignored for host queries. */
   uint32_t hash_slots;   /* launches that are not persistent: per-query seen-set slots (power of two);
                             0 = 2048, or with group 1 a bitmap of a collection of up to 131,072
-                            documents.  A full set only costs repeated work, never a different
-                            result */
+                            documents.  A set that is nearly full forgets: repeated work (and
+                            counters that vary with it), never a different result */
   uint32_t shape;        /* 0 or 1: one CTA per query (any k, any wave; the measured fastest);
                             2: one warp per query (k <= 128, wave 1, persistent, cta_warps
                             independent warps per CTA: 1/2/4, 0 = 4).  Both keep the

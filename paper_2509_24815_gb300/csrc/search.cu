@@ -141,7 +141,7 @@ struct Smem {
 };
 
 struct Shared {
-  uint32_t q, nzq, ncut, count, nvalid, hash_full, hash_n, bad;
+  uint32_t q, nzq, ncut, count, nvalid, hash_full, hash_n, crowded, bad;
   uint32_t ncand[2];  // candidates of a wave; waves take turns, so one may begin while another's count is still read
   float hf;
   uint32_t cut;
@@ -249,15 +249,22 @@ __device__ uint32_t merge_rank(const SearchArgs &a, Smem &s, Shared &sh, uint32_
   return min(k, cnt + nvalid);
 }
 
+// Sets sh.crowded once the hash set is three quarters full: by one thread, between a
+// wave's last barrier and the next one, so that it is the same for all of a wave's documents.
+__device__ __forceinline__ void note_crowded(const SearchArgs &a, const Smem &s, Shared &sh) {
+  if (!s.seen && sh.hash_n > a.HS / 4 * 3) sh.crowded = 1u;
+}
+
 // Makes the nc ranked entries the top-k; `done` also drops the wave's candidates.
 template <int NT>
-__device__ void merge_commit(Smem &s, Shared &sh, uint32_t nc, bool done) {
+__device__ void merge_commit(const SearchArgs &a, Smem &s, Shared &sh, uint32_t nc, bool done) {
   const int tid = threadIdx.x;
   for (uint32_t i = tid; i < nc; i += NT) { s.tk_s()[i] = s.tmp_s()[i]; s.tk_id()[i] = s.tmp_id()[i]; }
   if (tid == 0) {
     sh.count = nc;
     sh.nvalid = 0;
     if (done) sh.ncand[s.turn ^ 1u] = 0;
+    note_crowded(a, s, sh);
   }
   __syncthreads();
 }
@@ -283,7 +290,7 @@ __device__ void eval_wave(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, 
   // Software pipeline per lane group: the next document's (id, row) are loaded
   // while the current one is scored, and the seen-bitmap test is issued with
   // the row's loads and read after the dot (a seen document's score is dropped).
-  const bool crowded = sh.hash_n > a.HS / 4 * 3;
+  const bool crowded = sh.crowded != 0u;
   uint32_t dn = SEISMIC_NONE_ID;
   unsigned long long rn = 0ull;
   if ((uint32_t)grp < n) src.fetch(grp, dn, rn);
@@ -444,7 +451,7 @@ __device__ __forceinline__ void eval_wave_flat(const SearchArgs &a, Smem &s, Sha
   float2 *sums = reinterpret_cast<float2 *>(queue);
   const uint8_t *qf = s.qfilt();
   const uint32_t per = (n + NW - 1) / NW, rounds = (per + 31u) / 32u, dpw = (per + rounds - 1) / rounds;
-  const bool crowded = sh.hash_n > a.HS / 4 * 3;
+  const bool crowded = sh.crowded != 0u;
   const uint32_t mine = min(n, (warp + 1) * per);  // the warp's members: warp * per .. mine
   for (uint32_t r0 = warp * per; r0 < mine; r0 += dpw) {
     const uint32_t i = r0 + lane;
@@ -673,6 +680,10 @@ __device__ __forceinline__ uint32_t score(const SearchArgs &a, Smem &s, Shared &
   }
   const uint32_t m = sh.ncand[s.turn];
   s.turn ^= 1u;
+  if (!s.seen && m == 0) {  // no merge follows
+    if (threadIdx.x == 0) note_crowded(a, s, sh);
+    __syncthreads();
+  }
   return m;
 }
 
@@ -750,7 +761,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
     }
     if (tid < SEISMIC_STATS_N) sh.st[tid] = tid == SEISMIC_ST_T_START && a.stats ? globaltimer_ns() : 0ull;
     if (tid == 0) {
-      sh.count = 0; sh.ncand[0] = 0; sh.ncand[1] = 0; sh.nvalid = 0; sh.hash_full = 0; sh.hash_n = 0; sh.bad = 0;
+      sh.count = 0; sh.ncand[0] = 0; sh.ncand[1] = 0; sh.nvalid = 0; sh.hash_full = 0; sh.hash_n = 0; sh.crowded = 0; sh.bad = 0;
       sh.cut = a.cut;
       sh.hf = a.hf;
       if (a.q_cut) {  // learned per-query parameters (already validated by their producer)
@@ -853,7 +864,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
         for (uint32_t c0 = d0; c0 < d1; c0 += a.CAND) {
           const ListSrc src{nullptr, nullptr, 0u, c0, a.bdoc, a.bdoc_row};
           const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, d1 - c0), src, 0);
-          if (m) merge_commit<NT>(s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
+          if (m) merge_commit<NT>(a, s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
         }
         continue;
       }
@@ -964,7 +975,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
           if (m == 0) continue;
           const uint32_t nc = merge_rank<NT>(a, s, sh, m, false, 0, 0);
           if (G != 1 || be == first_end || nc < a.k || bscore(be - 1) >= limit(s.tmp_s()[a.k - 1])) {
-            merge_commit<NT>(s, sh, nc, true);
+            merge_commit<NT>(a, s, sh, nc, true);
             continue;
           }
           __syncthreads();  // everybody has read tmp
@@ -978,7 +989,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
             if (fk && bscore(done) < th) break;
             uint32_t nd;
             const uint32_t e = wave_end(done, be, fk, th, nd);
-            merge_commit<NT>(s, sh, merge_rank<NT>(a, s, sh, m, true, taken, taken + nd), false);
+            merge_commit<NT>(a, s, sh, merge_rank<NT>(a, s, sh, m, true, taken, taken + nd), false);
             taken += nd;
             done = e;
           }
@@ -1019,7 +1030,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
       for (uint32_t c0 = 0; c0 < total; c0 += a.CAND) {
         const NeighbourSrc src{stage ? s.clo() : nullptr, a.knn, a.fwd_row, stage ? 0u : a.seed[q], a.kappa, a.knn_bits, c0};
         const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, total - c0), src, stage);
-        if (m) merge_commit<NT>(s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
+        if (m) merge_commit<NT>(a, s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
       }
     }
 
