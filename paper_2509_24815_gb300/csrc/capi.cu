@@ -274,6 +274,7 @@ int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const
   while (a.BPOW2 < a.BMAX) a.BPOW2 <<= 1;
   a.HS = p->hash_slots ? p->hash_slots : 2048;
   a.CAND = kCand;
+  a.n_docs = ix->n_docs;
   if (p->learned) {
     // (cut, heap_factor) per query from the MLP, fused ahead of the search
     size_t need = (size_t)nq * (SEISMIC_MLP_IN * 4 + 8);
@@ -342,7 +343,7 @@ int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const
     // persistent CTAs keep a seen bitmap of the collection each, in global
     // memory (cleared per query), so deduplication never overflows
     int blocks = 1;
-    if ((rc = search_occupancy(group, nw, smem, &blocks))) return rc;
+    if ((rc = search_occupancy(a, group, nw, smem, &blocks))) return rc;
     grid = (uint32_t)std::min<uint64_t>(nq, (uint64_t)std::max(1, blocks) * sm_count(ix->device));
     a.seen_words = words;
     if ((rc = w->seen.ensure((size_t)grid * a.seen_words * 4))) return rc;

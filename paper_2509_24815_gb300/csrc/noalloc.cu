@@ -124,6 +124,7 @@ extern "C" int seismic_search_noalloc(seismic_index *ix, const seismic_csr *quer
   while (a.BPOW2 < a.BMAX) a.BPOW2 <<= 1;
   a.HS = 16;
   a.CAND = kCand;
+  a.n_docs = ix->n_docs;
   a.sum_absmax = ix->sum_absmax;
   a.prefetch = p->no_prefetch ? 0u : 256u;
   a.perm = nullptr;
@@ -132,7 +133,7 @@ extern "C" int seismic_search_noalloc(seismic_index *ix, const seismic_csr *quer
   const size_t smem = search_fit(a, group, p->cta_warps, 0u, (uint32_t)sms, 0u, nw);
   if (smem == 0) return fail(SEISMIC_EBUDGET, "search: shared memory per query exceeds 200 KB");
   int blocks = 1;
-  if ((rc = search_occupancy(group, nw, smem, &blocks))) return rc;
+  if ((rc = search_occupancy(a, group, nw, smem, &blocks))) return rc;
   uint64_t grid = std::min<uint64_t>(nq, (uint64_t)std::max(1, blocks) * sms);
   grid = std::min<uint64_t>(grid, cap_ctas);
   a.seen_words = (uint32_t)words;

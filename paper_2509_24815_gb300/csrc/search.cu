@@ -426,10 +426,10 @@ __device__ float warp_row(const SearchArgs &a, const Smem &s, unsigned long long
 // block visited: 2.94 to 1.93 ms.  A filter of 4096 bytes (4.6 candidates per
 // document instead of 3.6): 67.6 ms; of 16,384 bytes (3 CTAs per SM): 65.9 ms.
 // Prefetching the rows into L2 no longer pays (64.3 ms) and is gone here.
-template <int NT, bool FP16, class Src>
+template <int NT, bool FP16, bool SMALL, class Src>
 __device__ __forceinline__ void eval_wave_flat(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, const Src &src,
                                                int knn_stage) {
-  constexpr int U = FP16 ? 1 : 2, NW = NT / 32;
+  constexpr int U = FP16 || SMALL ? 1 : 2, NW = NT / 32;
   constexpr uint32_t kUnit = FP16 ? 2u * kUnitBytes : kUnitBytes;  // bytes of two chunks: their terms (fp16 rows: and values)
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, below = (1u << lane) - 1u;
   const bool full = sh.count == a.k;
@@ -669,12 +669,12 @@ __device__ __forceinline__ void eval_wave_flat(const SearchArgs &a, Smem &s, Sha
 }
 
 // Scores n documents of a source; returns the number of candidates (the same in every thread).
-template <int G, int NT, class Src>
+template <int G, int NT, bool SMALL, class Src>
 __device__ __forceinline__ uint32_t score(const SearchArgs &a, Smem &s, Shared &sh, uint32_t n, const Src &src,
                                           int knn_stage) {
   if constexpr (G == 1) {
-    if (a.fp16) eval_wave_flat<NT, true>(a, s, sh, n, src, knn_stage);
-    else eval_wave_flat<NT, false>(a, s, sh, n, src, knn_stage);
+    if (a.fp16) eval_wave_flat<NT, true, SMALL>(a, s, sh, n, src, knn_stage);
+    else eval_wave_flat<NT, false, SMALL>(a, s, sh, n, src, knn_stage);
   } else {
     eval_wave<G, NT>(a, s, sh, n, src, knn_stage);
   }
@@ -721,11 +721,12 @@ __device__ void bitonic_sort_u64(unsigned long long *keys, uint32_t P2) {
 }
 
 // Lane groups: 5 CTAs of 256 threads per SM (48 registers).  Group 1: 4 CTAs (64
-// registers, two groups of units in flight without spills worth naming, 46 KB of
-// shared memory each); 5 CTAs at 48 registers, one group in flight and half the
-// filter took 68.7 ms where 4 take 65.6 (1M documents, 10k queries, cut 10).
-template <int G, int NW>
-__global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
+// registers, two groups of units in flight, 46 KB of shared memory each).  SMALL:
+// 5 CTAs (48 registers, one group in flight), which took 69 ms where 4 take 64 (1M documents,
+// 10k queries, cut 10), but win in small collections, where most of a query is the
+// latency of its lists' block scores and first waves (search_fit).
+template <int G, int NW, bool SMALL>
+__global__ void __launch_bounds__(NW * 32, (G == 1 && !SMALL ? 1024 : 1280) / (NW * 32))
     k_search(const __grid_constant__ SearchArgs a) {
   constexpr int NT = NW * 32;
   __shared__ Shared sh;
@@ -863,7 +864,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
         }
         for (uint32_t c0 = d0; c0 < d1; c0 += a.CAND) {
           const ListSrc src{nullptr, nullptr, 0u, c0, a.bdoc, a.bdoc_row};
-          const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, d1 - c0), src, 0);
+          const uint32_t m = score<G, NT, SMALL>(a, s, sh, min(a.CAND, d1 - c0), src, 0);
           if (m) merge_commit<NT>(a, s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
         }
         continue;
@@ -971,7 +972,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
           const bool single = G != 1 && be - bi == 1;
           const ListSrc src{keys + bi, s.bptr(), single ? 0u : be - bi,
                             single ? s.bptr()[(uint32_t)(keys[bi] & 0xFFFFFFFFu)] + c0 : c0, a.bdoc, a.bdoc_row};
-          const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, ndocs - c0), src, 0);
+          const uint32_t m = score<G, NT, SMALL>(a, s, sh, min(a.CAND, ndocs - c0), src, 0);
           if (m == 0) continue;
           const uint32_t nc = merge_rank<NT>(a, s, sh, m, false, 0, 0);
           if (G != 1 || be == first_end || nc < a.k || bscore(be - 1) >= limit(s.tmp_s()[a.k - 1])) {
@@ -1029,7 +1030,7 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
       }
       for (uint32_t c0 = 0; c0 < total; c0 += a.CAND) {
         const NeighbourSrc src{stage ? s.clo() : nullptr, a.knn, a.fwd_row, stage ? 0u : a.seed[q], a.kappa, a.knn_bits, c0};
-        const uint32_t m = score<G, NT>(a, s, sh, min(a.CAND, total - c0), src, stage);
+        const uint32_t m = score<G, NT, SMALL>(a, s, sh, min(a.CAND, total - c0), src, stage);
         if (m) merge_commit<NT>(a, s, sh, merge_rank<NT>(a, s, sh, m, false, 0, 0), true);
       }
     }
@@ -1047,20 +1048,20 @@ __global__ void __launch_bounds__(NW * 32, (G == 1 ? 1024 : 1280) / (NW * 32))
   }
 }
 
-template <int G, int NW>
+template <int G, int NW, bool SMALL = false>
 int launch_t(const SearchArgs &a, size_t smem, uint32_t grid, cudaStream_t st) {
   static std::atomic<uint64_t> configured{0};
-  int rc = set_smem_limit_once(configured, (const void *)k_search<G, NW>, (int)kMaxSmem);
+  int rc = set_smem_limit_once(configured, (const void *)k_search<G, NW, SMALL>, (int)kMaxSmem);
   if (rc) return rc;
-  k_search<G, NW><<<grid, NW * 32, smem, st>>>(a);
+  k_search<G, NW, SMALL><<<grid, NW * 32, smem, st>>>(a);
   SZ_CUDA(cudaGetLastError());
   return SEISMIC_OK;
 }
 
-template <int G, int NW>
+template <int G, int NW, bool SMALL = false>
 int occupancy_t(size_t smem, int *blocks) {
-  SZ_CUDA(cudaFuncSetAttribute(k_search<G, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
-  SZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_search<G, NW>, NW * 32, smem));
+  SZ_CUDA(cudaFuncSetAttribute(k_search<G, NW, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+  SZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_search<G, NW, SMALL>, NW * 32, smem));
   return SEISMIC_OK;
 }
 
@@ -1151,6 +1152,10 @@ size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefe
       // CTAs 65.9 instead of 63.7
       a.CAND = w > nw ? kWideCand : kCand;
       if ((smem = search_layout(a, w)) <= kMaxSmem) {
+        // 8000 queries of 10..150 entries with 4 and with 5 CTAs per SM: 2000 documents 1.91 and 1.71 ms, 20,000 4.44 and
+        // 4.02, 50,000 (lists of 1000) 8.02 and 7.41; 1000 queries of 20,000 0.850 and 0.847.  Batches that
+        // 4 CTAs hold in two rounds gain nothing
+        a.small = w == 8 && smem <= kSmallSmem && a.n_docs <= kSmallDocs && a.nq > 8 * sms;
         nw = w;
         return smem;
       }
@@ -1166,6 +1171,7 @@ size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefe
 int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, uint32_t grid, cudaStream_t st) {
 #define SZ_CASE(G_, NW_) \
   if (group == G_ && nw == NW_) return launch_t<G_, NW_>(a, smem, grid, st);
+  if (a.small && group == 1 && nw == 8) return launch_t<1, 8, true>(a, smem, grid, st);
   SZ_CASE(1, 4) SZ_CASE(1, 8) SZ_CASE(1, 16) SZ_CASE(1, 32)
   SZ_CASE(8, 4) SZ_CASE(8, 8) SZ_CASE(8, 16)
   SZ_CASE(16, 4) SZ_CASE(16, 8) SZ_CASE(16, 16)
@@ -1174,9 +1180,10 @@ int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem,
   return fail(SEISMIC_EINVAL, "group must be 1/8/16/32 and cta_warps 4/8/16");
 }
 
-int search_occupancy(uint32_t group, uint32_t nw, size_t smem, int *blocks) {
+int search_occupancy(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, int *blocks) {
 #define SZ_CASE(G_, NW_) \
   if (group == G_ && nw == NW_) return occupancy_t<G_, NW_>(smem, blocks);
+  if (a.small && group == 1 && nw == 8) return occupancy_t<1, 8, true>(smem, blocks);
   SZ_CASE(1, 4) SZ_CASE(1, 8) SZ_CASE(1, 16) SZ_CASE(1, 32)
   SZ_CASE(8, 4) SZ_CASE(8, 8) SZ_CASE(8, 16)
   SZ_CASE(16, 4) SZ_CASE(16, 8) SZ_CASE(16, 16)

@@ -59,9 +59,10 @@ struct SearchArgs {
   // not traversed, the heap is seeded with the document and its graph row, and
   // the kappa-NN expansion follows (NULL: ordinary search)
   const uint32_t *seed;
-  // CTA kernel, group 1: documents are scored chunk by chunk by all threads
-  // of the CTA (a wave's chunks laid end to end, then summed per document)
+  // CTA kernel, group 1: each warp scores its own share of a wave's documents
   uint32_t flat;
+  uint32_t small;   // group 1 in CTAs of 8 warps: the build for five CTAs per SM
+  uint64_t n_docs;  // documents of the index (search_fit's rule)
   // shared-memory layout
   uint32_t W, QN, BMAX, BPOW2, HS, CAND;
   uint32_t NP;      // block-score partial arrays, one per warp that scores summaries
@@ -78,6 +79,8 @@ constexpr uint32_t kSeenDocs = 131072;   // collections up to here keep a launch
 constexpr uint32_t kFilter = 8192;        // bytes of the query's term filter
 constexpr uint32_t kWarpQueueBytes = 1536;  // a warp's candidate queue
 constexpr uint32_t kWarpDocsBytes = 960;   // a warp's document arrays
+constexpr uint32_t kSmallDocs = 65536;    // collections up to here run five CTAs of 8 warps per SM where they fit
+constexpr uint32_t kSmallSmem = 228u * 1024u / 5u - 1024u - 512u;  // dynamic shared memory of one of five CTAs
 constexpr uint32_t kShortChunks = 256;    // chunks of a row whose positions fit a queue entry (11 bits)
 constexpr uint32_t kMaxWave = 64;  // blocks per wave (CTA kernel)
 size_t search_layout(SearchArgs &a, uint32_t nw);
@@ -89,7 +92,7 @@ constexpr uint32_t kMaxSmem = 226u * 1024u;  // dynamic shared memory of a CTA, 
 // returns its size, or 0 when the query's data exceed 200 KB.
 size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefer, uint32_t sms, uint32_t bitmap_words,
                   uint32_t &nw);
-int search_occupancy(uint32_t group, uint32_t nw, size_t smem, int *blocks);
+int search_occupancy(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, int *blocks);
 size_t search_layout_warp(SearchArgs &a);
 int launch_search_warp(const SearchArgs &a, uint32_t group, size_t smem, uint32_t grid, uint32_t wpb,
                        cudaStream_t st);
