@@ -309,9 +309,10 @@ typedef struct {
   uint32_t max_batch;     /* requests per launch; 0 = 256 */
   uint32_t streams;       /* batches in flight at once (1..64); 0 = 4 */
   uint32_t max_query_nnz; /* admission: longer requests are refused; 0 = 1024 */
-  uint32_t slot_budget;   /* admission: requests on the device at once; 0 = what the search kernel's
-                             shared memory per query (query, block scores, a 100-entry heap) lets
-                             stay resident: CTAs per SM x SMs */
+  uint32_t slot_budget;   /* admission: requests on the device at once; 0 = three times what the search
+                             kernel's shared memory per query (query, block scores, a 100-entry
+                             heap) lets stay resident, CTAs per SM x SMs: a batch's slots are freed
+                             by its slowest query */
 } seismic_server_params;
 
 /* Creates a server over `index` (which must outlive it).  `search` fixes the

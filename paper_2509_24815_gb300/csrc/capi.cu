@@ -200,7 +200,7 @@ int check_params(const seismic_index *ix, const seismic_search_params *p) {
 
 int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const seismic_search_params *p,
               uint32_t *ids_out, float *scores_out, int32_t out_on_device, void *stream, uint64_t *stats,
-              const uint32_t *seed, uint32_t warps) {
+              const uint32_t *seed, uint32_t beside) {
   if (!ix || !queries || !w) return fail(SEISMIC_EINVAL, "NULL index/queries");
   int rc = check_params(ix, p);
   if (rc) return rc;
@@ -333,7 +333,7 @@ int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const
   // document (100k documents, 12.5 KB: 1000 queries 2.0 ms; the hash set 2.5)
   const uint32_t words = (uint32_t)(((ix->n_docs + 31) / 32 + 3) & ~3ull);
   uint32_t nw = 8;
-  const size_t smem = search_fit(a, group, p->cta_warps, warps, (uint32_t)sm_count(ix->device),
+  const size_t smem = search_fit(a, group, p->cta_warps, beside, (uint32_t)sm_count(ix->device),
                                  !a.persistent && !p->hash_slots && ix->n_docs <= kSeenDocs ? words : 0u, nw);
   if (smem == 0)
     return fail(SEISMIC_EBUDGET, "search: shared memory per query (" + std::to_string(a.budget) +

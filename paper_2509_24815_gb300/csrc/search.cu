@@ -1132,7 +1132,7 @@ static size_t search_budget(const SearchArgs &a, uint32_t nw) {
 // not depend on the choice.
 static uint32_t search_warps(uint32_t nq, uint32_t sms) { return nq > 4 * sms ? 8u : nq > sms ? 16u : 32u; }
 
-size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefer, uint32_t sms, uint32_t bitmap_words,
+size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t beside, uint32_t sms, uint32_t bitmap_words,
                   uint32_t &nw) {
   nw = asked ? asked : 8u;
   a.NP = nw;
@@ -1143,7 +1143,7 @@ size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefe
   size_t smem = 0;
   if (a.persistent) a.HS = 16;  // the seen set is a bitmap in global memory
   if (!a.flat) return search_layout(a, nw);
-  const uint32_t slots = a.HS, wide = asked ? asked : prefer ? prefer : search_warps(a.nq, sms);
+  const uint32_t slots = a.HS, wide = asked ? asked : search_warps(a.nq + beside, sms);
   for (int form = bitmap_words ? 0 : 1; form < 2; form++) {
     a.seen_words = form == 0 ? bitmap_words : 0u;
     a.HS = form == 0 ? bitmap_words : slots;
@@ -1155,7 +1155,7 @@ size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefe
         // 8000 queries of 10..150 entries with 4 and with 5 CTAs per SM: 2000 documents 1.91 and 1.71 ms, 20,000 4.44 and
         // 4.02, 50,000 (lists of 1000) 8.02 and 7.41; 1000 queries of 20,000 0.850 and 0.847.  Batches that
         // 4 CTAs hold in two rounds gain nothing
-        a.small = w == 8 && smem <= kSmallSmem && a.n_docs <= kSmallDocs && a.nq > 8 * sms;
+        a.small = w == 8 && smem <= kSmallSmem && a.n_docs <= kSmallDocs && a.nq + beside > 8 * sms;
         nw = w;
         return smem;
       }

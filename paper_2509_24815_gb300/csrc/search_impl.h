@@ -86,22 +86,22 @@ constexpr uint32_t kMaxWave = 64;  // blocks per wave (CTA kernel)
 size_t search_layout(SearchArgs &a, uint32_t nw);
 int launch_search(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, uint32_t grid, cudaStream_t st);
 constexpr uint32_t kMaxSmem = 226u * 1024u;  // dynamic shared memory of a CTA, beside a little static
-// Chooses warps per CTA (asked, else prefer, else by the number of queries), the seen set
+// Chooses warps per CTA (asked, else by the number of queries on the GPU, a.nq and `beside`), the seen set
 // (bitmap_words > 0: a bitmap in shared memory where it fits) and, for queries
 // too long for group 1's arrays, lane groups; lays shared memory out and
 // returns its size, or 0 when the query's data exceed 200 KB.
-size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t prefer, uint32_t sms, uint32_t bitmap_words,
+size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t beside, uint32_t sms, uint32_t bitmap_words,
                   uint32_t &nw);
 int search_occupancy(const SearchArgs &a, uint32_t group, uint32_t nw, size_t smem, int *blocks);
 size_t search_layout_warp(SearchArgs &a);
 int launch_search_warp(const SearchArgs &a, uint32_t group, size_t smem, uint32_t grid, uint32_t wpb,
                        cudaStream_t st);
 // One search call on a workspace (the C ABI's seismic_search, the server's
-// streams); `seed` selects the graph-refinement mode above, `warps` the warps per
-// CTA of group 1 where the parameters leave them open (results do not depend on it).
+// streams); `seed` selects the graph-refinement mode above, `beside` is the number of
+// queries of other calls on the GPU (for the launch configuration; results do not depend on it).
 int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const seismic_search_params *p,
               uint32_t *ids_out, float *scores_out, int32_t out_on_device, void *stream, uint64_t *stats,
-              const uint32_t *seed = nullptr, uint32_t warps = 0);
+              const uint32_t *seed = nullptr, uint32_t beside = 0);
 int search_occupancy_warp(uint32_t group, uint32_t k, size_t smem, uint32_t wpb, int *blocks);
 
 struct ExactArgs {

@@ -4,9 +4,9 @@
 // Requests queue on the host.  progress() reaps batches that finished on the
 // device and admits waiting requests as soon as a stream and enough device
 // slots are free, so new batches start while others are still running and
-// their work overlaps on the GPU.  Admission is bounded by a slot budget: the
-// number of queries the search kernel can hold resident at once, which its
-// shared memory per query (the query bitmap, block scores, the top-k heap of
+// their work overlaps on the GPU.  Admission is bounded by a slot budget: three
+// times the number of queries the search kernel can hold resident at once, which
+// its shared memory per query (the query bitmap, block scores, the top-k heap of
 // k entries) fixes through the occupancy calculator.  Each stream owns its
 // workspace and pinned staging buffers, so concurrent batches share nothing
 // but the read-only index; a query's result does not depend on what runs
@@ -58,12 +58,13 @@ template <class T> struct Pinned {
   }
 };
 
-// Warps per CTA where the search parameters leave them open.  A batch frees its
-// slots and its stream when its last query ends, so queries that end sooner,
-// fewer at a time, serve more of them: 4096 requests of mixed length and k over
-// 1M documents in 25.5 ms with 16 warps, 29 with 8 (27 before the warps scored
-// documents by themselves).
-constexpr uint32_t kServeWarps = 16;
+// Requests admitted per CTA that the GPU holds.  A batch frees its slots and its
+// stream when its last query ends, so with as many requests as CTAs most slots wait
+// for the slowest query of their batch.  Requests past the resident ones wait
+// on the device and start as CTAs end.  16,384 requests at once over 1M documents, at
+// 1, 2, 3 and 4.5 per CTA of 8 warps: 144k, 202k, 262k and 266k q/s (cut 5); 42k, 61k,
+// 80k and 86k (cut 10, graph, learned parameters); latencies below saturation do not depend on it.
+constexpr uint32_t kServeDepth = 3;
 
 struct Slot {
   cudaStream_t st = nullptr;
@@ -154,7 +155,7 @@ int launch_batch(seismic_server *srv, Slot &s) {
   p.k = k;
   p.max_query_nnz = srv->pp.max_query_nnz;
   if ((rc = search_ws(srv->ix, &s.ws, &q, &p, s.d_ids.as<uint32_t>(), s.d_sc.as<float>(), 1, s.st, nullptr,
-                      nullptr, kServeWarps)))
+                      nullptr, srv->inflight)))
     return rc;
   SZ_CUDA(cudaMemcpyAsync(s.h_ids.p, s.d_ids.p, (size_t)n * k * 4, cudaMemcpyDeviceToHost, s.st));
   SZ_CUDA(cudaMemcpyAsync(s.h_sc.p, s.d_sc.p, (size_t)n * k * 4, cudaMemcpyDeviceToHost, s.st));
@@ -234,7 +235,7 @@ int seismic_server_create(seismic_index *ix, const seismic_search_params *search
     if (!srv->pp.max_query_nnz) srv->pp.max_query_nnz = 1024;
     if (srv->pp.streams > 64) return fail(SEISMIC_EINVAL, "at most 64 streams");
     SZ_CUDA(cudaSetDevice(ix->device));
-    // slot budget: resident queries the search kernel's shared memory allows
+    // slot budget: from the resident queries the search kernel's shared memory allows
     uint32_t budget = srv->pp.slot_budget;
     if (!budget) {
       SearchArgs a{};
@@ -246,18 +247,16 @@ int seismic_server_create(seismic_index *ix, const seismic_search_params *search
       a.HS = 16;
       a.k = std::max<uint32_t>(search->k, 100);
       a.alpha_q = search->alpha_q;
-      const uint32_t nw = search->cta_warps ? search->cta_warps : 8, g = search->group ? search->group : 1;
       a.dim = ix->dim;
-      a.flat = g == 1 ? 1u : 0u;
-      a.CAND = kCand;
-      a.NP = nw;
-      size_t smem = search_layout(a, nw);
-      int blocks = 1;
-      int rc = search_occupancy(a, g, nw, smem, &blocks);
-      if (rc) return rc;
-      int sms = 1;
+      a.n_docs = ix->n_docs;
+      a.persistent = 1;
+      a.nq = 1u << 30;  // more than the GPU holds
+      uint32_t nw = 8, g = search->group ? search->group : 1;
+      int sms = 1, blocks = 1, rc;
       SZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ix->device));
-      budget = (uint32_t)std::max(1, blocks) * (uint32_t)sms;
+      const size_t smem = search_fit(a, g, search->cta_warps, 0u, (uint32_t)sms, 0u, nw);
+      if (smem && (rc = search_occupancy(a, g, nw, smem, &blocks))) return rc;  // (0: the search refuses such queries)
+      budget = kServeDepth * (uint32_t)std::max(1, blocks) * (uint32_t)sms;
     }
     srv->budget = budget;
     for (uint32_t i = 0; i < srv->pp.streams; i++) srv->slots.emplace_back();
@@ -288,7 +287,7 @@ int seismic_server_create(seismic_index *ix, const seismic_search_params *search
         p.k = kk;
         p.max_query_nnz = srv->pp.max_query_nnz;
         if ((rc = search_ws(ix, &s.ws, &q, &p, s.d_ids.as<uint32_t>(), s.d_sc.as<float>(), 1, s.st, nullptr,
-                            nullptr, kServeWarps)))
+                            nullptr, budget)))
           return rc;
         SZ_CUDA(cudaStreamSynchronize(s.st));
       }

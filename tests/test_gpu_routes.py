@@ -102,3 +102,32 @@ def test_default_launch_by_number_of_queries(sz, collection, kw, launch, nq):
     if "hash_slots" not in launch:  # a set that forgets scores some documents again
         for name in ("docs", "doc_nnz", "knn_docs", "knn_nnz"):
             np.testing.assert_array_equal(gst[:, sz.STATS.index(name)], rst[:, sz.STATS.index(name)], err_msg=name)
+
+
+# A server admits three requests per CTA that the GPU holds (9 per SM at least: three CTAs of 8 warps), so that a
+# batch's slowest query leaves no CTA idle, or what slot_budget says; results are those of the requests alone.
+@pytest.mark.parametrize("cta_warps", [0, 8])
+@pytest.mark.parametrize("budget", [0, 100])
+def test_server_admission(sz, collection, cta_warps, budget):
+    import torch
+    queries, ix = collection
+    p = sz.search_params(k=10, cut=8, heap_factor=0.8, wave=8, persistent=True, use_knn=True, cta_warps=cta_warps)
+    ids, sc = sz.seismic_search(ix, queries, p)
+    srv = sz.Server(ix, p, max_batch=128, streams=32, max_query_nnz=100, slot_budget=budget)
+    n = 4000
+    tickets = []
+    for i in range(n):
+        a, b = int(queries.indptr[i % queries.n_rows]), int(queries.indptr[i % queries.n_rows + 1])
+        tickets.append(srv.submit(queries.terms[a:b], queries.vals[a:b], 10))
+    srv.progress()  # admits
+    torch.cuda.synchronize()
+    done = srv.progress()  # what was admitted has ended
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert done == budget if budget else 9 * sms <= done < n
+    while done < n:
+        done += srv.progress()
+    for i, t in enumerate(tickets):
+        gi, gs, _ = srv.result(t, 10)
+        np.testing.assert_array_equal(gi, ids[i % queries.n_rows])
+        np.testing.assert_array_equal(gs, sc[i % queries.n_rows])
+    srv.close()
