@@ -18,11 +18,14 @@ import numpy as np
 
 from . import DeviceCSR, search_params, seismic_info, seismic_search
 
-# (shape, group, cta_warps, wave, L2 row prefetch): shape 1 = one CTA per query
+# (shape, group, cta_warps, wave, L2 prefetch): shape 1 = one CTA per query
 # (group 1: warp-local scoring, else lane groups of that width), 2 = one
-# warp per query
+# warp per query.  cta_warps 0 = the library's choice by the number of queries
+# (one query over 1M documents: 1.5 ms where 8 take 2.6, 16 take 1.9; large
+# batches: 8).  The prefetch is of member lists and, outside group 1, of rows.
 DEFAULT_CANDIDATES = tuple(
-    [(1, 1, 8, v, pf) for v in (4, 8, 16, 32) for pf in (False, True)] +
+    [(1, 1, 0, v, pf) for v in (4, 8, 16, 32) for pf in (False, True)] +
+    [(1, 1, 8, v, True) for v in (8, 16)] +
     [(1, 1, 16, v, pf) for v in (8, 16) for pf in (False, True)] +
     [(1, 8, 8, v, pf) for v in (4, 16) for pf in (False, True)] +
     [(1, 16, 8, 16, True), (1, 8, 4, 16, True)] +

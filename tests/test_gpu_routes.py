@@ -131,3 +131,14 @@ def test_server_admission(sz, collection, cta_warps, budget):
         np.testing.assert_array_equal(gi, ids[i % queries.n_rows])
         np.testing.assert_array_equal(gs, sc[i % queries.n_rows])
     srv.close()
+
+
+# The tuner times the launch that the library chooses by itself, and so returns none that is slower.
+def test_autotune_reaches_the_default_launch(sz, collection):
+    from paper_2509_24815_gb300 import autotune
+    queries, ix = collection
+    best, table = autotune.autotune(ix, sz.DeviceCSR.from_host(queries.slice(0, 1)), dict(k=10, cut=8, heap_factor=0.8))
+    own = [t["ms"] for t in table if t["shape"] == 1 and t["group"] == 1 and t["cta_warps"] == 0]
+    assert len(own) == 8
+    assert min(t["ms"] for t in table if "ms" in t) <= min(own)
+    assert {x: best[x] for x in ("k", "cut", "heap_factor")} == dict(k=10, cut=8, heap_factor=0.8)
