@@ -129,10 +129,10 @@ uint64_t splitmix64_next(uint64_t &state) {
 // sequential merge of the two sorted rows.  Argmax ties keep the lower
 // centroid index.
 constexpr int kAsgThreads = 128;
-constexpr int kAsgCC = 50;        // centroids per chunk (cluster index fits in u8); as many as leave 2 CTAs per SM
+// Centroids per chunk (asg_chunk): as many as leave two CTAs per SM.
 constexpr int kAsgMaxEnt = 8192;  // nonzeros per chunk (= kMaxRowNnzBuild bound below)
 static_assert(kMaxRowNnzBuild <= kAsgMaxEnt, "a centroid row must fit one chunk");
-static_assert((size_t)kAsgCC * kAsgThreads * 8 >= (size_t)(kAsgMaxEnt + 1) * 4, "the cursors share the accumulators");
+constexpr uint32_t kAsgMinCC = ((kAsgMaxEnt + 1) * 4 + kAsgThreads * 8 - 1) / (kAsgThreads * 8);  // the cursors share the accumulators
 
 __device__ __forceinline__ void asg_scan_rank(const uint32_t *bits, uint16_t *rank, uint32_t W, uint32_t *wtmp) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kAsgThreads / 32;
@@ -201,15 +201,15 @@ __global__ void __launch_bounds__(kAsgThreads) k_assign(
     const uint32_t *__restrict__ list_doc, const uint32_t *__restrict__ cent_ptr,
     const uint32_t *__restrict__ cent_doc, const uint64_t *__restrict__ indptr,
     const uint16_t *__restrict__ terms, const float *__restrict__ vals, uint32_t dim,
-    const unsigned long long *__restrict__ fwd_row, const uint8_t *__restrict__ fwd, int fp16,
+    const unsigned long long *__restrict__ fwd_row, const uint8_t *__restrict__ fwd, int fp16, uint32_t chunk,
     double *__restrict__ best, uint32_t *__restrict__ assign) {
   extern __shared__ __align__(16) unsigned char smem[];
   const uint32_t W = (dim + 31) / 32;
-  double *acc = reinterpret_cast<double *>(smem);                    // kAsgCC * kAsgThreads
+  double *acc = reinterpret_cast<double *>(smem);                    // chunk * kAsgThreads
   // the chunk's per-term counts and cursors (kAsgMaxEnt + 1) live in the
   // accumulators' space: they are dead once the chunk's index is built
   uint32_t *ccur = reinterpret_cast<uint32_t *>(smem);
-  float *ent_w = reinterpret_cast<float *>(acc + kAsgCC * kAsgThreads);  // kAsgMaxEnt
+  float *ent_w = reinterpret_cast<float *>(acc + chunk * kAsgThreads);  // kAsgMaxEnt
   uint32_t *cbits = reinterpret_cast<uint32_t *>(ent_w + kAsgMaxEnt);    // W
   uint16_t *coff = reinterpret_cast<uint16_t *>(cbits + W);               // kAsgMaxEnt + 1
   uint16_t *crank = coff + (kAsgMaxEnt + 1);                              // W
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kAsgThreads) k_assign(
     uint32_t c0 = 0;
     while (c0 < nb) {
       uint32_t c1 = c0, ent = 0;
-      while (c1 < nb && c1 - c0 < (uint32_t)kAsgCC) {
+      while (c1 < nb && c1 - c0 < chunk) {
         uint32_t cd = cent_doc[cp0 + c1];
         uint32_t len = (uint32_t)(indptr[cd + 1] - indptr[cd]);
         if (c1 > c0 && ent + len > (uint32_t)kAsgMaxEnt) break;
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kAsgThreads) k_assign(
         const uint32_t j = list_doc[lp0 + i];
         for (uint32_t cc = 0; cc < ncc; cc++) a[cc * kAsgThreads] = 0.0;
         // the member's terms in ascending order, 8 at a time with their values, the next 8 read while these
-        // are scored (read behind their terms, with 48 centroids per chunk: 0.43 s where this takes 0.39, 100k documents, 100 blocks)
+        // are scored (read behind their terms: 0.42 s where this takes 0.40, 100k documents, 100 blocks, 48 centroids per chunk)
         const unsigned long long row = fwd_row[j];
         const uint8_t *rec = fwd + (size_t)(uint32_t)row * kUnitBytes;
         const uint32_t nch = (uint32_t)(row >> 32), nnz = (uint32_t)(indptr[j + 1] - indptr[j]);
@@ -339,10 +339,19 @@ __global__ void __launch_bounds__(kAsgThreads) k_assign(
   }
 }
 
-size_t asg_smem_bytes(uint32_t dim) {
+size_t asg_smem_bytes(uint32_t dim, uint32_t chunk) {
   uint32_t W = (dim + 31) / 32;
-  return (size_t)kAsgCC * kAsgThreads * 8 + (size_t)kAsgMaxEnt * 4 + W * 4 + (size_t)(kAsgMaxEnt + 1) * 2 + W * 2 +
+  return (size_t)chunk * kAsgThreads * 8 + (size_t)kAsgMaxEnt * 4 + W * 4 + (size_t)(kAsgMaxEnt + 1) * 2 + W * 2 +
          kAsgMaxEnt + 16;
+}
+
+// As many centroids per chunk as leave two CTAs per SM (sm_bytes of shared memory, 1 KB of it reserved per CTA):
+// every chunk walks all members again, and a CTA alone on its SM waits for its own chains of fp64 additions
+// (100k documents, 100 blocks, 51 and 56 centroids: 0.39 s with two CTAs, 0.55 with one).  30,522 terms: 51,
+// 45,000: 48 (0.41 s; 0.55 with 50), 65,536: 44.
+uint32_t asg_chunk(uint32_t dim, size_t sm_bytes) {
+  const size_t rest = asg_smem_bytes(dim, 0) + 1024 + 256, half = sm_bytes / 2;
+  return std::max<uint32_t>(kAsgMinCC, half > rest ? (uint32_t)std::min<size_t>(255, (half - rest) / (kAsgThreads * 8)) : 0u);
 }
 
 }  // namespace
@@ -578,7 +587,10 @@ int build_index(const seismic_csr *docs, const seismic_build_params *bp, seismic
         (rc = upload(d_t, D.t)) || (rc = upload(d_v, D.v)) || (rc = d_best.alloc(npost * 8)) ||
         (rc = d_asg.alloc(npost * 4)))
       return rc;
-    size_t smem = asg_smem_bytes(d);
+    int sm_bytes = 0;
+    SZ_CUDA(cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ix->device));
+    const uint32_t chunk = asg_chunk(d, (size_t)sm_bytes);
+    const size_t smem = asg_smem_bytes(d, chunk);
     SZ_CUDA(cudaFuncSetAttribute(k_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int sms = 1;
     SZ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ix->device));
@@ -587,7 +599,7 @@ int build_index(const seismic_csr *docs, const seismic_build_params *bp, seismic
       k_assign<<<grid, kAsgThreads, smem>>>(d_work.as<uint32_t>(), (uint32_t)work.size(), d_lptr.as<uint32_t>(),
                                             d_ldoc.as<uint32_t>(), d_cptr.as<uint32_t>(), d_cdoc.as<uint32_t>(),
                                             d_ip.as<uint64_t>(), d_t.as<uint16_t>(), d_v.as<float>(), d,
-                                            ix->fwd_row.as<unsigned long long>(), ix->fwd_data.as<uint8_t>(), fp16,
+                                            ix->fwd_row.as<unsigned long long>(), ix->fwd_data.as<uint8_t>(), fp16, chunk,
                                             d_best.as<double>(), d_asg.as<uint32_t>());
       SZ_CUDA(cudaGetLastError());
       SZ_CUDA(cudaDeviceSynchronize());
