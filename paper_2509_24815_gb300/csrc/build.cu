@@ -348,7 +348,7 @@ size_t asg_smem_bytes(uint32_t dim, uint32_t chunk) {
 // As many centroids per chunk as leave two CTAs per SM (sm_bytes of shared memory, 1 KB of it reserved per CTA):
 // every chunk walks all members again, and a CTA alone on its SM waits for its own chains of fp64 additions
 // (100k documents, 100 blocks, 51 and 56 centroids: 0.39 s with two CTAs, 0.55 with one).  30,522 terms: 51,
-// 45,000: 48 (0.41 s; 0.55 with 50), 65,536: 44.
+// 45,000: 48 (0.41 s; 0.55 with 50), 65,535: 44.
 uint32_t asg_chunk(uint32_t dim, size_t sm_bytes) {
   const size_t rest = asg_smem_bytes(dim, 0) + 1024 + 256, half = sm_bytes / 2;
   return std::max<uint32_t>(kAsgMinCC, half > rest ? (uint32_t)std::min<size_t>(255, (half - rest) / (kAsgThreads * 8)) : 0u);

@@ -145,12 +145,12 @@ def test_autotune_reaches_the_default_launch(sz, collection):
 
 
 # The centroids that clustering takes at a time depend on the vocabulary's bitmap (56 at 500 terms, 51 at 30,522, 48 at
-# 45,000, 44 at 65,536): the clusters do not.
+# 45,000, 44 at 65,535): the clusters do not.
 def test_clusters_do_not_depend_on_the_vocabulary(sz):
     rng = np.random.default_rng(9)
     docs = _rows(4000, lambda i: rng.integers(0, 500, rng.integers(1, 40)), -2, 9, 500, rng)
     want = None
-    for dim in (500, 30522, 45000, 65536):
+    for dim in (500, 30522, 45000, 65535):
         ix = sz.seismic_build(synth.CSR(docs.indptr, docs.terms, docs.vals, dim), lambda_=300, beta=150, alpha=0.5, seed=4)
         got = [sz.seismic_export(ix, "cent"), sz.seismic_export(ix, "bdoc")]
         ix.close()
