@@ -25,7 +25,6 @@ from . import DeviceCSR, search_params, seismic_info, seismic_search
 # batches: 8).  The prefetch is of member lists and, outside group 1, of rows.
 DEFAULT_CANDIDATES = tuple(
     [(1, 1, 0, v, pf) for v in (4, 8, 16, 32) for pf in (False, True)] +
-    [(1, 1, 8, v, True) for v in (8, 16)] +
     [(1, 1, 16, v, pf) for v in (8, 16) for pf in (False, True)] +
     [(1, 8, 8, v, pf) for v in (4, 16) for pf in (False, True)] +
     [(1, 16, 8, 16, True), (1, 8, 4, 16, True)] +
