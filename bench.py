@@ -61,11 +61,19 @@ DEFAULT_WORKLOAD = "c3"
 RECALL_TARGET = 0.9
 K = 10
 METRIC = "QPS at recall@10>=0.9 (batched Seismic search, fixed parameters)"
-# DRAM traffic of k_search per byte it executes (read + write), from one ncu capture of the current
-# kernel on 300k documents (fp32 rows, cut 10, heap_factor 0.8, wave 8), keyed by the L2 prefetch (of
-# member lists; rows are read in units where they are needed); used to estimate a full launch's traffic
-# from its executed bytes.  A form without a capture of the current kernel reports null.
-TRAFFIC_PER_EXEC_BYTE = {True: (16.156699e9 + 0.916050e9) / 41.034674e9}
+# DRAM bytes of k_search (read + write, ncu) per byte of its work counters, by workload and form of the launch (group,
+# L2 prefetch; fp32 rows), captured at wave 8 (c2s, c2: cut 5; c3: cut 30 with the graph; heap_factor 0.9).  A form, or a
+# workload, without a capture of the current kernel reports null.
+TRAFFIC_PER_EXEC_BYTE = {("c2s", 1, True): (9.327395e9 + 0.529235e9) / 24.652338e9,
+                         ("c2", 1, True): (82.270126e9 + 6.408401e9) / 146.776087e9,
+                         ("c3", 1, True): (541.247271e9 + 40.613514e9) / 758.709090e9}
+
+
+def traffic_ratio(workload, launch):
+    """DRAM bytes per counted byte for this launch, or None without a capture of it."""
+    if launch["shape"] == 2:
+        return None
+    return TRAFFIC_PER_EXEC_BYTE.get((workload, launch["group"] or 1, not launch["no_prefetch"]))
 
 
 def log(*a):
@@ -424,7 +432,7 @@ def main():
     ap.add_argument("--no-compact", action="store_true", help="skip the fp16 forward-value form")
     ap.add_argument("--no-parity", action="store_true", help="skip the sampled oracle parity")
     ap.add_argument("--learn-target", type=float, default=0.9)
-    ap.add_argument("--prefetch", type=int, default=0, help="TMA L2 prefetch of the wave's rows (when not autotuned)")
+    ap.add_argument("--prefetch", type=int, default=0, help="TMA L2 prefetch of member lists and, outside group 1, rows (when not autotuned)")
     ap.add_argument("--autotune", type=int, default=1, help="tune the launch configuration at the operating point")
     ap.add_argument("--graph", type=int, default=1, help="time the step as a CUDA graph replay")
     args = ap.parse_args()
@@ -571,8 +579,7 @@ def main():
     alg_bytes = float(metrics.algorithmic_bytes(st1, K, w["quant"], w["kappa"], knn_bits=kbits).sum())
     _, _, stw = sz.seismic_search(ix, dq, p, stats=True)
     exec_bytes = float(metrics.algorithmic_bytes(stw, K, w["quant"], w["kappa"], knn_bits=kbits).sum())
-    slots = 152 * 5 if launch["shape"] != 2 else 152 * 16
-    occupancy = metrics.queue_occupancy(stw, slots)
+    occupancy = metrics.queue_occupancy(stw, metrics.resident_queries(stw))
     log(f"bytes per launch: method (wave 1) {alg_bytes / 1e9:.2f} GB, executed (wave {launch['wave']}) "
         f"{exec_bytes / 1e9:.2f} GB; queue occupancy {occupancy}")
 
@@ -639,7 +646,7 @@ def main():
     peak, peak_kind = peaks()
     sec = float(np.mean(per)) * 1e-3
     achieved = alg_bytes / sec / 1e9  # this rank's kernel, per launch
-    ratio = TRAFFIC_PER_EXEC_BYTE.get(not launch["no_prefetch"]) if launch["shape"] != 2 else None
+    ratio = traffic_ratio(args.workload, launch)
     traffic = ratio * exec_bytes if ratio else None
     line = {
         "metric": METRIC,
@@ -658,8 +665,10 @@ def main():
                      "alg_bytes_per_launch": alg_bytes, "alg_bytes_basis": "work counters of the sequential "
                      "visiting order (wave 1) at the operating point",
                      "executed_bytes_per_launch": exec_bytes, "executed_frac": exec_bytes / sec / 1e9 / peak,
-                     "traffic_basis": ("ncu DRAM bytes per executed byte on the 300k-document workload (same "
-                                       "prefetch setting), scaled by this launch's executed bytes") if traffic else None,
+                     "executed_bytes_basis": "work counters of the timed wave; documents scored ahead of the "
+                     "threshold and undone are not in them",
+                     "traffic_basis": "ncu DRAM bytes per counted byte of this workload's launch (same group and "
+                     "prefetch setting), times this launch's counted bytes" if traffic else None,
                      "traffic_over_alg": (traffic / alg_bytes) if traffic else None},
         "queue_occupancy": occupancy,
         "e2e": {"value": e2e_qps, "unit": "queries/s", "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h)},

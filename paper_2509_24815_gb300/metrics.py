@@ -47,6 +47,18 @@ def algorithmic_bytes(stats: np.ndarray, k: int, quantized: bool, kappa: int = 0
     return b
 
 
+def resident_queries(stats: np.ndarray) -> int:
+    """The most queries that were on the device at once, from the per-query
+    device timestamps: the CTAs (or warps) that a persistent launch keeps
+    resident, once it has as many queries as that."""
+    t0 = stats[:, STATS.index("t_start_ns")].astype(np.int64)
+    t1 = stats[:, STATS.index("t_end_ns")].astype(np.int64)
+    t = np.concatenate([t0, t1])
+    step = np.concatenate([np.ones(len(t0), dtype=np.int64), -np.ones(len(t1), dtype=np.int64)])
+    order = np.lexsort((step, t))  # an end at a start's time comes first: the next query on the same slot
+    return int(np.cumsum(step[order]).max(initial=0))
+
+
 def queue_occupancy(stats: np.ndarray, slots: int) -> dict:
     """Load balance of one persistent launch from the per-query device
     timestamps: `busy` = the fraction of slot-time (slots = resident CTAs or
