@@ -18,7 +18,7 @@
 // update, a barrier), so the next two terms' postings are loaded ahead.  With
 // the accumulators in global memory (n_docs floats per CTA, cleared before and
 // after each query, every posting a scattered read-modify-write in L2 or DRAM)
-// 1000 queries over 100,000 documents took 5.4 ms; here 0.67 ms (one query of 40 entries over 1M documents: 4.1 ms, here 0.12).
+// 1000 queries over 100,000 documents took 5.35 ms; here 0.71 ms (one query of 40 entries over 1M documents: 4.1 ms, here 0.12).
 #include "search_impl.h"
 
 namespace seismic {
@@ -295,15 +295,40 @@ __global__ void __launch_bounds__(kExNT) k_exact_join(const ExactArgs a) {
 
 }  // namespace
 
+// Fewer queries than about one and a half times the CTAs that run at once (slots): several CTAs share a query's tiles.
+// Least of the rounds of CTAs times a CTA's documents; a tile's barriers count as 13,000 more (152 queries, 100,000
+// documents: 3 tiles of 20,000 each 191 us, 4 of 14,286 210), a CTA's first bound on the k-th best as 4000; the
+// smaller tiles only where they win.  100,000 documents, queries of 10..150 entries, with tiles of 24,576
+// and as many splits as all run at once, and here: 10 queries 103 and 96 us, 200 queries 378 and 286, 400 queries 555 and 483.
+static void ex_split(ExactArgs &a, uint32_t least, uint32_t most, uint32_t slots) {
+  a.tiles = least;
+  a.splits = 1;
+  if (2ull * a.nq >= 3ull * slots) return;
+  uint64_t best = ~0ull;
+  for (uint32_t tiles : {least, most}) {
+    const uint64_t docs = (a.n_docs + tiles - 1) / tiles;
+    for (uint32_t s = 1; s <= std::min(tiles, std::max(1u, 4u * slots / a.nq)); s++) {
+      if (s > 1 && (uint64_t)a.nq * s * a.k > (uint64_t)slots * kExactMaxK) break;  // the splits' results
+      const uint64_t cost = ((uint64_t)a.nq * s + slots - 1) / slots * ((tiles + s - 1) / s * (docs + 13000u) + 4000u);
+      if (cost < best) {
+        best = cost;
+        a.tiles = tiles;
+        a.splits = s;
+      }
+    }
+  }
+}
+
 // Working memory: the bounds table, the claim words and the splits' results; it
 // depends on the index only, so it is allocated once.
 size_t exact_layout(ExactArgs &a, uint32_t sms, void *base) {
-  a.tiles = (a.n_docs + ex_tile(a.k) - 1) / ex_tile(a.k);
+  const uint32_t least = (a.n_docs + ex_tile(a.k) - 1) / ex_tile(a.k);
+  const uint32_t most = (a.n_docs + ex_tile(kExactMaxK) - 1) / ex_tile(kExactMaxK);
+  ex_split(a, least, most, kExCtas * sms);
   a.tile = (a.n_docs + a.tiles - 1) / a.tiles;
   a.area = ex_area(a.k);
   a.sms = sms;
   const size_t claim = ((size_t)a.dim * 4 + 255) & ~(size_t)255;
-  const uint32_t most = (a.n_docs + ex_tile(kExactMaxK) - 1) / ex_tile(kExactMaxK);
   const size_t bounds = ((size_t)a.dim * (most + 1) * 4 + 255) & ~(size_t)255;
   unsigned char *p = reinterpret_cast<unsigned char *>(base);
   a.claim = reinterpret_cast<uint32_t *>(p);
@@ -314,8 +339,6 @@ size_t exact_layout(ExactArgs &a, uint32_t sms, void *base) {
 
 int launch_exact(ExactArgs a, cudaStream_t st) {
   if (a.k == 0 || a.k > kExactMaxK) return fail(SEISMIC_EINVAL, "exact search: k must be in 1..1024");
-  // fewer queries than CTAs that run at once: several CTAs share a query's tiles, as many as all run at once
-  a.splits = std::max(1u, std::min(a.tiles, kExCtas * a.sms / a.nq));
   const size_t smem = ex_smem(a.k, a.tile);
   static std::atomic<uint64_t> configured{0}, configured2{0};
   int rc;
