@@ -292,7 +292,7 @@ int search_ws(seismic_index *ix, Workspace *w, const seismic_csr *queries, const
     a.q_hf = qh;
     a.QN = std::max<uint32_t>(a.QN, 32);
   }
-  // defaults: one CTA per query with chunk-flattened scoring (the measured fastest)
+  // defaults: one CTA per query whose warps score their own documents (the measured fastest)
   uint32_t group = p->group ? p->group : (p->shape == 2 ? 8 : 1);
   a.sum_absmax = ix->sum_absmax;
   a.prefetch = p->no_prefetch ? 0u : 256u;

@@ -49,7 +49,7 @@ using namespace dev;
 // quarters full stops probing: a document takes its slot whatever is there, so a lookup
 // stays one atomic, and what was there is forgotten.  (Few documents are met
 // twice -- 3 % of a search of 34,000 -- so forgetting costs little, while 16 probes
-// per document made one query over 1M documents take 2.4 ms instead of 1.8.)
+// per document make one query over 1M documents take 2.7 ms instead of 1.5.)
 __device__ __forceinline__ bool seen_insert(uint32_t *tab, uint32_t hs_mask, uint32_t d, bool crowded, uint32_t *full) {
   const uint32_t key = d + 1u;
   uint32_t h = (d * 0x9E3779B1u) & hs_mask;
@@ -1156,7 +1156,7 @@ size_t search_fit(SearchArgs &a, uint32_t &group, uint32_t asked, uint32_t besid
     a.seen_words = form == 0 ? bitmap_words : 0u;
     a.HS = form == 0 ? bitmap_words : slots;
     for (uint32_t w : {wide, nw}) {
-      // wide CTAs score more documents at once: one query 1.45 ms instead of 1.77, but batches of 8-warp
+      // wide CTAs score more documents at once: one query 1.49 ms instead of 1.82, but batches of 8-warp
       // CTAs 65.9 instead of 63.7
       a.CAND = w > nw ? kWideCand : kCand;
       if ((smem = search_layout(a, w)) <= kMaxSmem) {

@@ -53,7 +53,7 @@ struct SearchArgs {
   // on |summary value| (fixes the fixed-point scale of the summary scores)
   uint32_t warp_bytes;
   float sum_absmax;
-  uint32_t prefetch;  // rows of the next block prefetched into L2 (at most this many; 0 = off)
+  uint32_t prefetch;  // nonzero: member lists and, outside group 1, rows (warp shape: at most this many) are prefetched into L2
   const uint32_t *perm;  // persistent launches pull queries in this order (NULL: 0, 1, 2, ...)
   // graph refinement (CTA kernel): query q is document seed[q]; its lists are
   // not traversed, the heap is seeded with the document and its graph row, and
