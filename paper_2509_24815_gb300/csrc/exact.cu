@@ -19,6 +19,8 @@
 // the accumulators in global memory (n_docs floats per CTA, cleared before and
 // after each query, every posting a scattered read-modify-write in L2 or DRAM)
 // 1000 queries over 100,000 documents took 5.35 ms; here 0.71 ms (one query of 40 entries over 1M documents: 4.1 ms, here 0.12).
+#include <cmath>
+
 #include "search_impl.h"
 
 namespace seismic {
@@ -299,17 +301,20 @@ __global__ void __launch_bounds__(kExNT) k_exact_join(const ExactArgs a) {
 // Least of the rounds of CTAs times a CTA's documents; a tile's barriers count as 13,000 more (152 queries, 100,000
 // documents: 3 tiles of 20,000 each 191 us, 4 of 14,286 210), a CTA's first bound on the k-th best as 4000; the
 // smaller tiles only where they win.  100,000 documents, queries of 10..150 entries, with tiles of 24,576
-// and as many splits as all run at once, and here: 10 queries 103 and 96 us, 200 queries 378 and 286, 400 queries 555 and 483.
+// and as many splits as all run at once, and here: 10 queries 103 and 96 us, 67 queries 177 and 141, 200 queries 378 and 287,
+// 400 queries 555 and 484.
 static void ex_split(ExactArgs &a, uint32_t least, uint32_t most, uint32_t slots) {
   a.tiles = least;
   a.splits = 1;
   if (2ull * a.nq >= 3ull * slots) return;
-  uint64_t best = ~0ull;
+  double best = 1e300;
   for (uint32_t tiles : {least, most}) {
-    const uint64_t docs = (a.n_docs + tiles - 1) / tiles;
+    const double docs = (double)((a.n_docs + tiles - 1) / tiles);
     for (uint32_t s = 1; s <= std::min(tiles, std::max(1u, 4u * slots / a.nq)); s++) {
       if (s > 1 && (uint64_t)a.nq * s * a.k > (uint64_t)slots * kExactMaxK) break;  // the splits' results
-      const uint64_t cost = ((uint64_t)a.nq * s + slots - 1) / slots * ((tiles + s - 1) / s * (docs + 13000u) + 4000u);
+      const double x = (double)a.nq * s / slots;  // rounds: a last one that is not full costs its part and a third of the rest
+      const double rounds = x <= 1.0 ? 1.0 : x + (std::ceil(x) - x) / 3.0, per = x <= 1.0 ? (tiles + s - 1) / s : (double)tiles / s;
+      const double cost = rounds * (per * (docs + 13000.0) + 4000.0);
       if (cost < best) {
         best = cost;
         a.tiles = tiles;
