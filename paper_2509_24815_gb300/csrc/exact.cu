@@ -312,9 +312,11 @@ static void ex_split(ExactArgs &a, uint32_t least, uint32_t most, uint32_t slots
     const double docs = (double)((a.n_docs + tiles - 1) / tiles);
     for (uint32_t s = 1; s <= std::min(tiles, std::max(1u, 4u * slots / a.nq)); s++) {
       if (s > 1 && (uint64_t)a.nq * s * a.k > (uint64_t)slots * kExactMaxK) break;  // the splits' results
-      const double x = (double)a.nq * s / slots;  // rounds: a last one that is not full costs its part and a third of the rest
+      // rounds: a last one that is not full costs its part and a third of the rest; past one they have to win by a tenth
+      // (50 queries of 40 entries, 1M documents: 6 parts 0.455 ms, 12 in two rounds 0.510)
+      const double x = (double)a.nq * s / slots;
       const double rounds = x <= 1.0 ? 1.0 : x + (std::ceil(x) - x) / 3.0, per = x <= 1.0 ? (tiles + s - 1) / s : (double)tiles / s;
-      const double cost = rounds * (per * (docs + 13000.0) + 4000.0);
+      const double cost = (x <= 1.0 ? 1.0 : 1.1) * rounds * (per * (docs + 13000.0) + 4000.0);
       if (cost < best) {
         best = cost;
         a.tiles = tiles;
